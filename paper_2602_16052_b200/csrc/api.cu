@@ -253,6 +253,7 @@ int run_layer(moespec_layer *L, const void *hidden, int M, int k, int B, void *o
   c.res_count = L->desc.resident_count;
   if (L->use_tc) {
     c.ru = tc_rows_per_unit(L->desc, M, k, c.B);
+    c.ru_down = tc_rows_per_down_unit(c.ru);
     c.early = tc_early_start(*desc, M) ? 1 : 0;
     c.dense_all = tc_dense_all(*desc, M) ? 1 : 0;
     // The early units follow the shortlist's rank order.  Router-based ranks follow the tokens' own
@@ -262,6 +263,9 @@ int run_layer(moespec_layer *L, const void *hidden, int M, int k, int B, void *o
       const int nS = c.B < L->ws.n_static ? c.B : L->ws.n_static;
       if ((long long)M * k < 4LL * nS) c.early = 0;
     }
+  } else {
+    c.ru = kCcUnitCols;
+    c.ru_down = kCcUnitDown;
   }
   c.debug_spin_limit = L->debug_spin_limit;
   c.debug_ready_bias = L->debug_ready_bias;
@@ -276,8 +280,10 @@ int run_layer(moespec_layer *L, const void *hidden, int M, int k, int B, void *o
   if ((e = mark(++launches)) != cudaSuccess) return cuda_fail(e);
   if ((e = launch_route_after_router(c)) != cudaSuccess) return cuda_fail(e);
   if ((e = mark(++launches)) != cudaSuccess) return cuda_fail(e);
-  if (!c.dense_all) {      // (trees of at most 16 tokens need no gathered rows on the tensor-core path)
-    if ((e = launch_gather(c, hidden)) != cudaSuccess) return cuda_fail(e);
+  // Trees of at most 16 tokens need no gathered rows on the tensor-core path.  The CUDA-core kernel fetches rows
+  // from hidden by itself; it needs this launch only where the rows are still to be worked out (large trees).
+  if (L->use_tc ? !c.dense_all : M > kMaxTokChunk) {
+    if ((e = launch_gather(c, L->use_tc ? hidden : nullptr)) != cudaSuccess) return cuda_fail(e);
     if ((e = mark(++launches)) != cudaSuccess) return cuda_fail(e);
   }
   if (L->use_tc) {
@@ -285,11 +291,7 @@ int run_layer(moespec_layer *L, const void *hidden, int M, int k, int B, void *o
     if ((e = launch_ffn_tensor_core(c, &L->maps, hidden, out)) != cudaSuccess) return cuda_fail(e);
     if ((e = mark(++launches)) != cudaSuccess) return cuda_fail(e);
   } else {
-    for (int phase = 0; phase < 2; ++phase) {
-      if ((e = launch_ffn_cuda_core(c, phase)) != cudaSuccess) return cuda_fail(e);
-      if ((e = mark(++launches)) != cudaSuccess) return cuda_fail(e);
-    }
-    if ((e = launch_combine(c, hidden, out)) != cudaSuccess) return cuda_fail(e);
+    if ((e = launch_ffn_cuda_core(c, &L->maps, hidden, out)) != cudaSuccess) return cuda_fail(e);
     if ((e = mark(++launches)) != cudaSuccess) return cuda_fail(e);
   }
   L->last_M = M;
@@ -374,7 +376,6 @@ int moespec_layer_create(const moespec_layer_desc *desc, moespec_layer_t **out_l
   }
   carve(d, L->R_cap, static_cast<char *>(L->arena), &L->ws);
   if (!use_tc) {
-    // the CUDA-core FFN stages a row of d (gate/up) or f (down) floats in shared memory
     bool fits = true;
     e = cc_configure(d, &fits);
     if (e != cudaSuccess || !fits) {
@@ -383,10 +384,10 @@ int moespec_layer_create(const moespec_layer_desc *desc, moespec_layer_t **out_l
       return e != cudaSuccess ? cuda_fail(e) : MOESPEC_ERR_UNSUPPORTED;
     }
   }
-  if (use_tc) {
+  {
     int cu_res = 0;
     e = tc_encode_maps(L->desc, L->ws, L->R_cap, &L->maps, &cu_res);
-    if (e == cudaSuccess) e = tc_configure();
+    if (e == cudaSuccess && use_tc) e = tc_configure();
     if (e == cudaSuccess) e = routing_configure();
     if (e != cudaSuccess) {
       cudaFree(L->arena);
@@ -623,7 +624,10 @@ int moespec_route_from_logits(moespec_layer_t *L, const float *logits, int M, in
   if (guard.err != cudaSuccess) return cuda_fail(guard.err);
   LaunchCtx c{&L->desc, &L->ws, M, k, B > L->desc.n_experts ? L->desc.n_experts : B, L->R_cap,
               static_cast<cudaStream_t>(stream), 0};
-  if (L->use_tc) c.ru = tc_rows_per_unit(L->desc, M, k, c.B);
+  if (L->use_tc) {
+    c.ru = tc_rows_per_unit(L->desc, M, k, c.B);
+    c.ru_down = tc_rows_per_down_unit(c.ru);
+  }
   c.res_first = L->desc.resident_first;
   c.res_count = L->desc.resident_count;
   cudaError_t e = launch_route(c, logits);

@@ -1,0 +1,597 @@
+// CUDA-core expert FFN and combine: E_i(x) = W2 (silu(W1 x) * (W3 x)) on the routed rows with full-precision fp32
+// FMAs, then the gate-weighted outer sum.  This is the kernel of the fp32 configuration (a tensor-core tf32 product
+// would drop mantissa bits), of 16-bit layers whose widths the tensor-core kernel does not take, and a second
+// implementation for the others that shares nothing with it.
+//
+// One persistent launch.  What bounds it: the kept experts' weights have to come from HBM once (806 MB at d = 2048,
+// f = 1024, 32 experts: 123 us at 6.55 TB/s) and every routed row costs 3*d*f FMAs (504 rows: 90 us of the 148 SMs'
+// FMA pipes, more with the rows padded to a thread tile).  A kernel with one CTA per (row, 64 outputs) reads the
+// weights of an expert again for every row it has: 925 us there.  Here a work unit is 64 weight rows (32 gate and the
+// same 32 up rows, or 64 down rows) against a chunk of an expert's routed rows, so weights are read from HBM once and
+// from shared memory by a thread tile of 8 weight rows x up to 8 token rows (16 16-byte loads per 256 FMAs, which is
+// where the shared-memory and the FMA rates meet).
+//
+//   warps 0-3  producers: warp 0 draws units from the dispenser in list order (gate/up units first; a down unit waits,
+//              bounded, until the gate/up units of its rows are published).  A ring of stages takes 64-element K
+//              slices: the weight rows by TMA (one lane, two to four boxes; copied 16 bytes at a time by one warp they
+//              took longer than the products: 580 us), the token rows by cp.async, in gather order straight from
+//              `hidden` (with one warp 400 us, with four 320: a layer of 348 us instead of 925).  No gathered copy is
+//              read.  (At 64 rows per expert the products run at 30 TFLOP/s; a register-only outer product of the
+//              same shape reaches 51 on this part.)
+//   warps 4-11 two groups of 32 weight rows x four shares.  The shares split K when the chunk has at most 16 rows,
+//              K and rows when it has up to 32, rows up to 64, so that a thread's tile is never much wider than
+//              the rows there are.  Four lanes of a warp split K further (a 16-byte load each).  A thread's chain of
+//              additions is cut every 64 terms and the partial sums meet in a fixed tree, so the result does not
+//              depend on the schedule and its error is that of 64-term chains.  Then the unit's results are stored
+//              and published, and after the last unit the CTA waits (bounded) for all down units and takes its share
+//              of the combine.
+#include "internal.h"
+
+namespace moespec {
+
+namespace {
+
+constexpr int kCcWarps = 8;                            // consumer warps
+constexpr int kCcConsumers = kCcWarps * 32;
+constexpr int kCcProducerWarps = 4;
+constexpr int kCcThreads = (kCcProducerWarps + kCcWarps) * 32;
+// Registers: 384 threads are launched with 168 each (64512); 128 * 56 + 256 * 224 = 64512 after the split.
+constexpr int kCcRegsProducer = 56, kCcRegsConsumer = 224;
+constexpr int kCcK = 64;                               // K elements per stage
+constexpr int kCcRows = 64;                            // token rows of a unit's pass
+constexpr int kCcStages = 6;
+constexpr int kCcQueue = 4;
+constexpr int kCcRedPitch = 80;                        // floats per token row of the reduction buffer (64 + pad)
+constexpr int kCcRedBytes = 64 * kCcRedPitch * 4;      // K shares x token rows <= 64
+constexpr long long kCcSpinCycles = 2000000000LL;      // default bound of every wait: ~1 s at 2 GHz
+
+struct CcMaps {              // [experts, rows, K] as boxes of 128 bytes x 32 (gate, up) or 64 (down) rows
+  CUtensorMap w_gate, w_up, w_down;
+};
+
+struct CcArgs {
+  const Unit *units;
+  const int *n_units;        // [0] gate/up units, [1] down units
+  int *unit_counter;         // [0] dispenser, [1] finished down units
+  int *ready;                // per (expert, token chunk): finished gate/up units
+  int tiles_up;              // value of ready[] that releases a chunk's down units
+  int tiles_real;            // gate/up units per chunk
+  const void *hidden;        // [M, d]
+  void *x_perm;              // [R, d] gathered copy (written for inspection, not read)
+  void *h_mid;               // [R, f]
+  float *y;                  // [R, d]
+  const int *perm_row2tok;
+  const float *gate_w;       // [M, k]
+  const int *tokslot2row, *assign_idx;
+  void *out;
+  int *status;
+  int M, k, d, f, residual;
+  int res_first, res_count;  // res_count > 0: expert-parallel shard
+  long long spin_limit;
+};
+
+// one unit's pass over at most kCcRows rows
+struct CcPass {
+  int expert;                // -1: no more units
+  int tile, row0, n_rows, chunk, phase, last;     // last: the unit's final pass
+};
+
+__device__ __forceinline__ uint32_t cc_smem(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void cc_bar_init(uint32_t bar, uint32_t count) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
+}
+__device__ __forceinline__ void cc_bar_arrive(uint32_t bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ bool cc_bar_try(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+// Bounded wait.  Returns false when the CTA is aborting or the limit expired.
+__device__ __forceinline__ bool cc_bar_wait(uint32_t bar, uint32_t parity, volatile int *abort_flag, long long limit) {
+  if (cc_bar_try(bar, parity)) return true;
+  const long long t0 = clock64();
+  for (uint32_t i = 1;; ++i) {
+    if (cc_bar_try(bar, parity)) return true;
+    if ((i & 255u) == 0u) {
+      if (*abort_flag) return false;
+      if (clock64() - t0 > limit) {
+        *abort_flag = 1;
+        return false;
+      }
+    }
+  }
+}
+__device__ __forceinline__ int cc_ld_acquire(const int *p) {
+  int v;
+  asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void cc_red_release(int *p) {
+  asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(p) : "memory");
+}
+__device__ __forceinline__ void cc_copy16(uint32_t dst, const void *src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cc_copies_arrive(uint32_t bar) {
+  asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void cc_expect_tx(uint32_t bar, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
+// weights are read once per call: they leave L2 first
+__device__ __forceinline__ void cc_tma_3d(uint32_t dst, const CUtensorMap *map, uint32_t bar, int c0, int c1, int c2,
+                                          uint64_t policy) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%3, %4, %5}], [%2], %6;"
+      ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "l"(policy)
+      : "memory");
+}
+__device__ __forceinline__ void cc_consumers_bar() { asm volatile("bar.sync 1, %0;" ::"n"(kCcConsumers) : "memory"); }
+// Barrier of the consumer warps that tells every one of them whether any has given up a wait: they leave together.
+__device__ __forceinline__ bool cc_consumers_any(bool failed) {
+  uint32_t any;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.u32 p, %1, 0;\n\t"
+      "bar.red.or.pred q, 2, %2, p;\n\t"
+      "selp.u32 %0, 1, 0, q;\n\t}"
+      : "=r"(any)
+      : "r"((uint32_t)failed), "n"(kCcConsumers)
+      : "memory");
+  return any != 0;
+}
+
+// four consecutive elements as floats
+__device__ __forceinline__ float4 cc_load4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
+__device__ __forceinline__ float4 cc_load4(const __nv_bfloat16 *p) {
+  const uint2 raw = *reinterpret_cast<const uint2 *>(p);
+  const __nv_bfloat162 *h = reinterpret_cast<const __nv_bfloat162 *>(&raw);
+  const float2 a = __bfloat1622float2(h[0]), b = __bfloat1622float2(h[1]);
+  return make_float4(a.x, a.y, b.x, b.y);
+}
+__device__ __forceinline__ float4 cc_load4(const __half *p) {
+  const uint2 raw = *reinterpret_cast<const uint2 *>(p);
+  const __half2 *h = reinterpret_cast<const __half2 *>(&raw);
+  const float2 a = __half22float2(h[0]), b = __half22float2(h[1]);
+  return make_float4(a.x, a.y, b.x, b.y);
+}
+__device__ __forceinline__ void cc_store(float *p, float v) { *p = v; }
+__device__ __forceinline__ void cc_store(__nv_bfloat16 *p, float v) { *p = __float2bfloat16_rn(v); }
+__device__ __forceinline__ void cc_store(__half *p, float v) { *p = __float2half_rn(v); }
+__device__ __forceinline__ void cc_store4(float *p, float4 v) { *reinterpret_cast<float4 *>(p) = v; }
+__device__ __forceinline__ void cc_store4(__nv_bfloat16 *p, float4 v) {
+  __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
+  uint2 raw;
+  raw.x = *reinterpret_cast<uint32_t *>(&lo);
+  raw.y = *reinterpret_cast<uint32_t *>(&hi);
+  *reinterpret_cast<uint2 *>(p) = raw;
+}
+__device__ __forceinline__ void cc_store4(__half *p, float4 v) {
+  __half2 lo = __floats2half2_rn(v.x, v.y), hi = __floats2half2_rn(v.z, v.w);
+  uint2 raw;
+  raw.x = *reinterpret_cast<uint32_t *>(&lo);
+  raw.y = *reinterpret_cast<uint32_t *>(&hi);
+  *reinterpret_cast<uint2 *>(p) = raw;
+}
+
+// Weight slices lie in boxes of 128 bytes per row (two boxes for an fp32 slice, one for a 16-bit one) with the
+// 128-byte swizzle: 16-byte piece p of row r is at p ^ (r & 7).  The four weight-row lanes of a warp take rows
+// 0, 4, 2, 6 (+ 0 or 1, + 8 n), so that the rows which one shared-memory phase reads (two for fp32, four for 16-bit
+// types) fall into different banks.  Token rows lie plainly: a phase reads one of them.
+__device__ __forceinline__ int cc_lane_row(int lw) { return ((lw & 1) << 2) | (lw & 2); }
+
+template <typename T> constexpr int kCcRowBytes = kCcK * (int)sizeof(T);
+template <typename T> constexpr int kCcBoxes = kCcRowBytes<T> / 128;      // boxes along a row's slice
+template <typename T> constexpr int kCcStageBytes = (64 + kCcRows) * kCcRowBytes<T>;
+template <typename T> constexpr size_t kCcSmemBytes = (size_t)kCcStages * kCcStageBytes<T> + kCcRedBytes + 1024 + 1024;
+
+// The consumer warps' part of one pass: XT token rows per thread, XG row groups (1, 2, 4) and 4 / XG K shares.
+// Leaves the partial sums of every K share in red[share][token row][weight row].  Returns false when aborting.
+template <typename T, int XT, int XG>
+__device__ __forceinline__ bool cc_products(const uint8_t *stages, uint32_t bar_full, uint32_t bar_empty, uint32_t &it,
+                                            int n_stages_unit, int phase, float *red, volatile int *abort_flag,
+                                            long long limit) {
+  constexpr int KG = 4 / XG;
+  const int lane = threadIdx.x & 31, cw = (threadIdx.x >> 5) - kCcProducerWarps;
+  const int lk = lane & 3, lx = lane >> 4;
+  const int wg = cw & 1, share = cw >> 1;
+  const int xgi = share % XG, kgi = share / XG;
+  const int x_row = xgi * 2 * XT + lx;
+  // gate/up: rows 0..31 of the stage are gate rows, 32..63 the up rows of the same columns, and group wg takes 16 of
+  // each; down: group wg takes rows 32 * wg ..
+  const int r_lane = cc_lane_row((lane >> 2) & 3), w_lo = phase == 0 ? wg * 16 : wg * 32,
+            w_hi = phase == 0 ? 32 + wg * 16 : w_lo + 16;
+  float acc[8][XT], tot[8][XT];
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+#pragma unroll
+    for (int j = 0; j < XT; ++j) acc[i][j] = tot[i][j] = 0.f;
+  constexpr int kFlush = 4 * KG - 1;          // 64 terms of a thread's chain = 4 * KG stages
+  for (int s = 0; s < n_stages_unit; ++s, ++it) {
+    const uint32_t slot = it % kCcStages, ph = (it / kCcStages) & 1u;
+    if (!cc_bar_wait(bar_full + 8 * slot, ph, abort_flag, limit)) return false;
+    const uint8_t *w = stages + (size_t)slot * kCcStageBytes<T>;
+    const T *x = reinterpret_cast<const T *>(w + 64 * kCcRowBytes<T>) + x_row * kCcK + lk * 4;
+    // the token rows of the next block are on their way while this one's products are formed
+    float4 xv[2][XT];
+#pragma unroll
+    for (int j = 0; j < XT; ++j) xv[0][j] = cc_load4(x + 2 * j * kCcK + kgi * 16);
+#pragma unroll
+    for (int q = 0; q < XG; ++q) {
+      const int b = kgi + q * KG;
+      if (q + 1 < XG) {
+#pragma unroll
+        for (int j = 0; j < XT; ++j) xv[(q + 1) & 1][j] = cc_load4(x + 2 * j * kCcK + (b + KG) * 16);
+      }
+      // this lane's four elements: byte offset inside the 64-element slice, split into box, 16-byte piece and rest
+      const int off = (b * 16 + lk * 4) * (int)sizeof(T), piece = (off >> 4) & 7;
+      const uint8_t *wb = w + (off >> 7) * (64 * 128) + (off & 15);
+      const uint8_t *w0 = wb + r_lane * 128 + ((piece ^ r_lane) << 4);                  // the lane's even and odd rows
+      const uint8_t *w1 = wb + (r_lane + 1) * 128 + ((piece ^ (r_lane + 1)) << 4);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const float4 wv = cc_load4(reinterpret_cast<const T *>(((i & 1) ? w1 : w0) +
+                                                               ((i < 4 ? w_lo : w_hi) + 8 * ((i >> 1) & 1)) * 128));
+#pragma unroll
+        for (int j = 0; j < XT; ++j) acc[i][j] = fmaf(wv.x, xv[q & 1][j].x, acc[i][j]);
+#pragma unroll
+        for (int j = 0; j < XT; ++j) acc[i][j] = fmaf(wv.y, xv[q & 1][j].y, acc[i][j]);
+#pragma unroll
+        for (int j = 0; j < XT; ++j) acc[i][j] = fmaf(wv.z, xv[q & 1][j].z, acc[i][j]);
+#pragma unroll
+        for (int j = 0; j < XT; ++j) acc[i][j] = fmaf(wv.w, xv[q & 1][j].w, acc[i][j]);
+      }
+    }
+    __syncwarp();
+    if (lane == 0) cc_bar_arrive(bar_empty + 8 * slot);
+    if ((s & kFlush) == kFlush || s == n_stages_unit - 1) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j < XT; ++j) {
+          tot[i][j] += acc[i][j];
+          acc[i][j] = 0.f;
+        }
+    }
+  }
+  // The four K lanes: each keeps half of the weight rows after every exchange, lane lk ends with row pair
+  // 2 * (lk & 1) + (lk >> 1) of its four: stage rows base + 8 * (lk >> 1) + r_lane + {0, 1}, base = w_lo or w_hi.
+  const bool hi1 = lk & 1, hi2 = lk & 2;
+#pragma unroll
+  for (int j = 0; j < XT; ++j) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const float keep = hi1 ? tot[i + 4][j] : tot[i][j], send = hi1 ? tot[i][j] : tot[i + 4][j];
+      tot[i][j] = keep + __shfl_xor_sync(0xffffffffu, send, 1);
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const float keep = hi2 ? tot[i + 2][j] : tot[i][j], send = hi2 ? tot[i][j] : tot[i + 2][j];
+      tot[i][j] = keep + __shfl_xor_sync(0xffffffffu, send, 2);
+    }
+    float *dst = red + (size_t)(kgi * XG * 2 * XT + x_row + 2 * j) * kCcRedPitch + (hi1 ? w_hi : w_lo) + (hi2 ? 8 : 0) + r_lane;
+    *reinterpret_cast<float2 *>(dst) = make_float2(tot[0][j], tot[1][j]);
+  }
+  return true;
+}
+
+template <typename T, typename TO>
+__global__ void __launch_bounds__(kCcThreads, 1) ffn_cc_kernel(const __grid_constant__ CcMaps maps, CcArgs a) {
+  extern __shared__ uint8_t cc_smem_raw[];
+  uint8_t *stages = cc_smem_raw + ((1024u - (cc_smem(cc_smem_raw) & 1023u)) & 1023u);
+  float *red = reinterpret_cast<float *>(stages + kCcStages * kCcStageBytes<T>);
+  uint8_t *ctrl = stages + kCcStages * kCcStageBytes<T> + kCcRedBytes;
+  const uint32_t bar_full = cc_smem(ctrl), bar_empty = bar_full + 8 * kCcStages;
+  const uint32_t bar_q_full = bar_empty + 8 * kCcStages, bar_q_empty = bar_q_full + 8 * kCcQueue;
+  volatile int *abort_flag = reinterpret_cast<volatile int *>(ctrl + 16 * kCcStages + 16 * kCcQueue);
+  CcPass *queue = reinterpret_cast<CcPass *>(ctrl + 256);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+
+  pdl_trigger();
+  // The first ticket is drawn before the wait: the router kernel, which zeroes the dispenser, has completed before
+  // the routing kernel releases this one.
+  int t_first = 0;
+  if (threadIdx.x == 0) {
+    t_first = atomicAdd(a.unit_counter, 1);
+    for (int s = 0; s < kCcStages; ++s) {
+      cc_bar_init(bar_full + 8 * s, kCcProducerWarps * 32 + 1);      // the producers' copies, the announced bytes
+      cc_bar_init(bar_empty + 8 * s, kCcWarps);
+    }
+    for (int q = 0; q < kCcQueue; ++q) {
+      cc_bar_init(bar_q_full + 8 * q, 1);
+      cc_bar_init(bar_q_empty + 8 * q, kCcWarps + kCcProducerWarps - 1);
+    }
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncthreads();
+  pdl_wait();
+  const int n_up = a.n_units[0], n_down = a.n_units[1];
+
+  if (warp < kCcProducerWarps) {
+    // ------------------------------------------------------------------ producers
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kCcRegsProducer));
+    uint64_t wpol;
+    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(wpol));
+    uint32_t it = 0, qi = 0;
+    constexpr int kPieces = kCcRowBytes<T> / 16;          // 16-byte pieces of a row's slice
+    constexpr int kStep = 32 / kPieces * kCcProducerWarps;      // rows copied per round by the four warps
+    constexpr int kRounds = kCcRows / kStep;
+    const int piece = lane % kPieces, r_first = warp * (32 / kPieces) + lane / kPieces;
+    int next = t_first, pass = 0;                         // warp 0, lane 0: the unit drawn and the next pass over it
+    Unit un{};
+    bool ok = true;
+    while (true) {
+      const uint32_t q = qi % kCcQueue, qph = (qi / kCcQueue) & 1u;
+      ++qi;
+      if (warp == 0) {
+        if (lane == 0) {
+          const bool have = next < n_up + n_down;
+          if (have && pass == 0) un = a.units[next];
+          if (have && pass == 0 && un.phase == 1) {       // its rows of h_mid: every gate/up unit of the chunk
+            const long long t0 = clock64();
+            while (cc_ld_acquire(a.ready + un.chunk) < a.tiles_up) {
+              if (*abort_flag || clock64() - t0 > a.spin_limit) { *abort_flag = 1; ok = false; break; }
+              __nanosleep(32);
+            }
+          }
+          ok = ok && cc_bar_wait(bar_q_empty + 8 * q, qph ^ 1u, abort_flag, a.spin_limit);
+          if (ok) {
+            const int n = min(kCcRows, un.n_rows - pass * kCcRows);
+            const bool last = (pass + 1) * kCcRows >= un.n_rows;
+            queue[q] = CcPass{have ? un.expert : -1, un.tile, un.row0 + pass * kCcRows, n, un.chunk, un.phase, last};
+            cc_bar_arrive(bar_q_full + 8 * q);
+            ++pass;
+            if (have && last) {
+              pass = 0;
+              next = atomicAdd(a.unit_counter, 1);
+            }
+          }
+        }
+        __syncwarp();
+        ok = __shfl_sync(0xffffffffu, ok, 0);
+      } else {
+        ok = __all_sync(0xffffffffu, cc_bar_wait(bar_q_full + 8 * q, qph, abort_flag, a.spin_limit));
+      }
+      if (!ok) break;
+      const CcPass ps = queue[q];          // (warp 0 reads its own entry: it is the one that will replace it)
+      __syncwarp();
+      if (warp != 0 && lane == 0) cc_bar_arrive(bar_q_empty + 8 * q);
+      if (ps.expert < 0) break;
+      const int K = ps.phase == 0 ? a.d : a.f, n = ps.n_rows, e = ps.expert - a.res_first;
+      // where this lane's token rows come from: the token's hidden state (gate/up), or the row of h_mid (down)
+      const T *xbase = (ps.phase == 0 ? (const T *)a.hidden : (const T *)a.h_mid + (size_t)ps.row0 * a.f) +
+                       piece * (16 / sizeof(T));
+      int src[kRounds];
+#pragma unroll
+      for (int u = 0; u < kRounds; ++u) {
+        const int r = r_first + u * kStep;
+        src[u] = r < n ? (ps.phase == 0 ? a.perm_row2tok[ps.row0 + r] : r) * K : -1;
+      }
+      for (int k0 = 0; k0 < K; k0 += kCcK, ++it) {
+        const uint32_t slot = it % kCcStages, ph = (it / kCcStages) & 1u;
+        ok = __all_sync(0xffffffffu, cc_bar_wait(bar_empty + 8 * slot, ph ^ 1u, abort_flag, a.spin_limit));
+        if (!ok) break;
+        const uint32_t full = bar_full + 8 * slot;
+        const uint32_t ws = cc_smem(stages) + slot * kCcStageBytes<T>, xs = ws + 64 * kCcRowBytes<T>;
+        if (threadIdx.x == 0) {
+          cc_expect_tx(full, 64 * kCcRowBytes<T>);
+#pragma unroll
+          for (int h = 0; h < kCcBoxes<T>; ++h) {
+            const uint32_t dst = ws + h * (64 * 128);
+            const int col = k0 + h * (128 / (int)sizeof(T));
+            if (ps.phase == 0) {
+              cc_tma_3d(dst, &maps.w_gate, full, col, ps.tile * 32, e, wpol);
+              cc_tma_3d(dst + 32 * 128, &maps.w_up, full, col, ps.tile * 32, e, wpol);
+            } else {
+              cc_tma_3d(dst, &maps.w_down, full, col, ps.tile * 64, e, wpol);
+            }
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < kRounds; ++u)
+          if (src[u] >= 0) cc_copy16(xs + (r_first + u * kStep) * kCcRowBytes<T> + piece * 16, xbase + (src[u] + k0));
+        cc_copies_arrive(full);
+      }
+      if (!ok) break;
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    if (!ok && warp == 0) {      // giving up: the boxes on their way land before the CTA may leave (bounded)
+      const uint32_t lo = it > (uint32_t)kCcStages ? it - kCcStages : 0u;
+      for (uint32_t j = lo; j < it; ++j) {
+        const long long t0 = clock64();
+        while (!cc_bar_try(bar_full + 8 * (j % kCcStages), (j / kCcStages) & 1u))
+          if (clock64() - t0 > a.spin_limit) break;
+      }
+    }
+  } else {
+    // ------------------------------------------------------------------ consumers
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kCcRegsConsumer));
+    const int ct = threadIdx.x - kCcProducerWarps * 32;
+    uint32_t it = 0, qi = 0;
+    while (true) {
+      const uint32_t q = qi % kCcQueue, qph = (qi / kCcQueue) & 1u;
+      ++qi;
+      bool ok = cc_bar_wait(bar_q_full + 8 * q, qph, abort_flag, a.spin_limit);
+      const CcPass ps = queue[q];
+      __syncwarp();
+      if (lane == 0) cc_bar_arrive(bar_q_empty + 8 * q);
+      const int K = ps.phase == 0 ? a.d : a.f, n = ps.n_rows;
+      // row groups and rows per thread: 8 weight rows x XT token rows per thread, 2 * XT rows per group
+      const int xg = n <= 16 ? 1 : n <= 32 ? 2 : 4;
+      const int xt = (n + 2 * xg - 1) / (2 * xg);
+#define MOESPEC_CC(G, X)                                                                                            \
+  case G * 16 + X:                                                                                                  \
+    ok = cc_products<T, X, G>(stages, bar_full, bar_empty, it, K / kCcK, ps.phase, red, abort_flag, a.spin_limit);  \
+    break;
+      switch (ok && ps.expert >= 0 ? xg * 16 + xt : 0) {
+        MOESPEC_CC(1, 1) MOESPEC_CC(1, 2) MOESPEC_CC(1, 3) MOESPEC_CC(1, 4)
+        MOESPEC_CC(1, 5) MOESPEC_CC(1, 6) MOESPEC_CC(1, 7) MOESPEC_CC(1, 8)
+        MOESPEC_CC(2, 5) MOESPEC_CC(2, 6) MOESPEC_CC(2, 7) MOESPEC_CC(2, 8)
+        MOESPEC_CC(4, 5) MOESPEC_CC(4, 6) MOESPEC_CC(4, 7) MOESPEC_CC(4, 8)
+      }
+#undef MOESPEC_CC
+      if (cc_consumers_any(!ok) || ps.expert < 0) break;     // (behind this barrier all partial sums are written)
+      const int kg = 4 / xg, share_rows = xg * 2 * xt;
+      if (ps.phase == 0) {
+        const int col = ct & 31;
+        T *dst = (T *)a.h_mid + (size_t)ps.row0 * a.f + ps.tile * 32 + col;
+        for (int r = ct >> 5; r < n; r += kCcConsumers / 32) {
+          float g = 0.f, u = 0.f;
+          for (int s = 0; s < kg; ++s) {
+            g += red[(size_t)(s * share_rows + r) * kCcRedPitch + col];
+            u += red[(size_t)(s * share_rows + r) * kCcRedPitch + 32 + col];
+          }
+          cc_store(dst + (size_t)r * a.f, (g / (1.f + expf(-g))) * u);
+        }
+        // this unit's share of the gathered copy
+        const int pieces = a.d / (16 / (int)sizeof(T));
+        const int lo = pieces * ps.tile / a.tiles_real, w = pieces * (ps.tile + 1) / a.tiles_real - lo;
+        for (int i = ct; i < n * w; i += kCcConsumers) {
+          const int r = i / w, c = lo + i - r * w;
+          reinterpret_cast<uint4 *>((T *)a.x_perm + (size_t)(ps.row0 + r) * a.d)[c] =
+              reinterpret_cast<const uint4 *>((const T *)a.hidden + (size_t)a.perm_row2tok[ps.row0 + r] * a.d)[c];
+        }
+      } else {
+        const int col = ct & 63;
+        float *dst = a.y + (size_t)ps.row0 * a.d + ps.tile * 64 + col;
+        for (int r = ct >> 6; r < n; r += kCcConsumers / 64) {
+          float v = 0.f;
+          for (int s = 0; s < kg; ++s) v += red[(size_t)(s * share_rows + r) * kCcRedPitch + col];
+          dst[(size_t)r * a.d] = v;
+        }
+      }
+      cc_consumers_bar();             // the unit's stores precede its publication; the buffer is free again
+      if (ct == 0 && ps.last) cc_red_release(ps.phase == 0 ? a.ready + ps.chunk : a.unit_counter + 1);
+    }
+
+    // ---------------------------------------------------------------- combine
+    // out_t = sum over the kept slots of wgt[t, slot] * y[row(t, slot)], slots in a fixed order (outer sums of Eq. 2 /
+    // 7 / 8); exact zeros for a token with no kept expert (Section 3.3).  One warp per 128 columns of a token.
+    if (ct == 0 && !*abort_flag) {
+      const long long t0 = clock64();
+      while (cc_ld_acquire(a.unit_counter + 1) < n_down) {
+        if (clock64() - t0 > a.spin_limit) { *abort_flag = 1; break; }
+        __nanosleep(32);
+      }
+    }
+    __syncwarp();
+    if (cc_consumers_any(*abort_flag != 0)) {
+      if (ct == 0) atomicExch(a.status, (int)MOESPEC_ERR_TIMEOUT);
+      return;
+    }
+    const int k = a.k, d = a.d, slices = (d + 127) / 128, n_items = a.M * slices;
+    for (int item = (int)blockIdx.x + (ct >> 5) * (int)gridDim.x; item < n_items; item += kCcWarps * (int)gridDim.x) {
+      const int t = item / slices, c = (item - t * slices) * 128 + lane * 4;
+      int my_row = lane < k ? a.tokslot2row[(size_t)t * k + lane] : -1;
+      const float my_w = lane < k ? a.gate_w[(size_t)t * k + lane] : 0.f;
+      if (a.res_count > 0 && my_row >= 0) {      // expert-parallel shard: only the slots of resident experts
+        const int e = a.assign_idx[(size_t)t * k + lane];
+        if (e < a.res_first || e >= a.res_first + a.res_count) my_row = -1;
+      }
+      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int s0 = 0; s0 < k; s0 += 8) {
+        float4 v[8];
+        float w[8];
+        bool live[8];
+#pragma unroll
+        for (int s = 0; s < 8; ++s) {
+          const int row = __shfl_sync(0xffffffffu, my_row, (s0 + s) & 31);
+          w[s] = __shfl_sync(0xffffffffu, my_w, (s0 + s) & 31);
+          live[s] = s0 + s < k && row >= 0 && c < d;
+          v[s] = live[s] ? __ldcg(reinterpret_cast<const float4 *>(a.y + (size_t)row * d + c))
+                         : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+#pragma unroll
+        for (int s = 0; s < 8; ++s) {
+          if (live[s]) {
+            acc.x = fmaf(w[s], v[s].x, acc.x);
+            acc.y = fmaf(w[s], v[s].y, acc.y);
+            acc.z = fmaf(w[s], v[s].z, acc.z);
+            acc.w = fmaf(w[s], v[s].w, acc.w);
+          }
+        }
+      }
+      if (c < d) {
+        if (a.residual) {
+          const float4 h = cc_load4((const T *)a.hidden + (size_t)t * d + c);
+          acc.x += h.x; acc.y += h.y; acc.z += h.z; acc.w += h.w;
+        }
+        cc_store4((TO *)a.out + (size_t)t * d + c, acc);
+      }
+    }
+  }
+}
+
+template <typename T, typename TO>
+cudaError_t launch_cc(const LaunchCtx &c, const CcMaps &m, const CcArgs &a) {
+  return launch_kernel(ffn_cc_kernel<T, TO>, dim3(tc_grid_size(c.desc->device)), dim3(kCcThreads), kCcSmemBytes<T>,
+                       c.stream, m, a);
+}
+
+template <typename T, typename TO>
+cudaError_t configure_cc() {
+  return cudaFuncSetAttribute(ffn_cc_kernel<T, TO>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCcSmemBytes<T>);
+}
+
+}  // namespace
+
+// Widths whose fp32 row would not fit the opt-in shared memory of a block are not covered (*fits = false).
+cudaError_t cc_configure(const moespec_layer_desc &D, bool *fits) {
+  int optin = 0;
+  cudaError_t e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, D.device);
+  if (e != cudaSuccess) return e;
+  *fits = (size_t)D.d * sizeof(float) <= (size_t)optin && (size_t)D.f * sizeof(float) <= (size_t)optin;
+  if (!*fits) return cudaSuccess;
+  const bool same = D.out_dtype == 0 || D.out_dtype == D.dtype;
+  if (D.dtype == MOESPEC_BF16)
+    return same ? configure_cc<__nv_bfloat16, __nv_bfloat16>() : configure_cc<__nv_bfloat16, float>();
+  if (D.dtype == MOESPEC_FP16) return same ? configure_cc<__half, __half>() : configure_cc<__half, float>();
+  return configure_cc<float, float>();
+}
+
+cudaError_t launch_ffn_cuda_core(const LaunchCtx &c, const TcMaps *maps, const void *hidden, void *out) {
+  const moespec_layer_desc &D = *c.desc;
+  const Workspace &ws = *c.ws;
+  CcMaps m;
+  m.w_gate = maps->w_gate[2];
+  m.w_up = maps->w_up[2];
+  m.w_down = maps->w_down[1];
+  CcArgs a;
+  a.units = ws.units;
+  a.n_units = ws.counters + 3;
+  a.unit_counter = ws.unit_counter;
+  a.ready = ws.ready;
+  a.tiles_real = D.f / c.ru;
+  a.tiles_up = a.tiles_real + c.debug_ready_bias;
+  a.hidden = hidden;
+  a.x_perm = ws.x_perm;
+  a.h_mid = ws.h_mid;
+  a.y = ws.y;
+  a.perm_row2tok = ws.perm_row2tok;
+  a.gate_w = ws.gate_w;
+  a.tokslot2row = ws.tokslot2row;
+  a.assign_idx = ws.assign_idx;
+  a.out = out;
+  a.status = ws.status;
+  a.M = c.M; a.k = c.k; a.d = D.d; a.f = D.f;
+  a.residual = D.residual;
+  a.res_first = c.res_first;
+  a.res_count = c.res_count > 0 && c.res_count < D.n_experts ? c.res_count : 0;
+  a.spin_limit = c.debug_spin_limit > 0 ? c.debug_spin_limit : kCcSpinCycles;
+  const bool same = D.out_dtype == 0 || D.out_dtype == D.dtype;
+  if (D.dtype == MOESPEC_BF16)
+    return same ? launch_cc<__nv_bfloat16, __nv_bfloat16>(c, m, a) : launch_cc<__nv_bfloat16, float>(c, m, a);
+  if (D.dtype == MOESPEC_FP16) return same ? launch_cc<__half, __half>(c, m, a) : launch_cc<__half, float>(c, m, a);
+  return launch_cc<float, float>(c, m, a);
+}
+
+}  // namespace moespec

@@ -839,20 +839,23 @@ cudaError_t tc_encode_maps(const moespec_layer_desc &d, const Workspace &ws, int
   cudaError_t e = get_encode_fn(&enc);
   if (e != cudaSuccess) return e;
   const cuuint32_t ones[3] = {1, 1, 1};
-  const CUtensorMapDataType tm_dtype =
-      d.dtype == MOESPEC_FP16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
+  const CUtensorMapDataType tm_dtype = d.dtype == MOESPEC_FP16   ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16
+                                       : d.dtype == MOESPEC_BF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16
+                                                                 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
+  const cuuint64_t eb = (cuuint64_t)dtype_bytes(d.dtype);
+  const cuuint32_t box_k = (cuuint32_t)(128 / eb);       // a box row is one 128-byte swizzle row
   auto weights = [&](CUtensorMap *m, const void *base, int rows, int K, int box_rows) -> CUresult {
     cuuint64_t dims[3] = {(cuuint64_t)K, (cuuint64_t)rows, (cuuint64_t)(d.resident_count > 0 ? d.resident_count : d.n_experts)};
-    cuuint64_t strides[2] = {(cuuint64_t)K * 2, (cuuint64_t)rows * K * 2};
-    cuuint32_t box[3] = {kChunkK, (cuuint32_t)box_rows, 1};
+    cuuint64_t strides[2] = {(cuuint64_t)K * eb, (cuuint64_t)rows * K * eb};
+    cuuint32_t box[3] = {box_k, (cuuint32_t)box_rows, 1};
     return enc(m, tm_dtype, 3, const_cast<void *>(base), dims, strides, box, ones,
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   };
   auto rows2d = [&](CUtensorMap *m, void *base, int K, int box_rows) -> CUresult {
     cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)R_cap};
-    cuuint64_t strides[1] = {(cuuint64_t)K * 2};
-    cuuint32_t box[2] = {kChunkK, (cuuint32_t)box_rows};
+    cuuint64_t strides[1] = {(cuuint64_t)K * eb};
+    cuuint32_t box[2] = {box_k, (cuuint32_t)box_rows};
     return enc(m, tm_dtype, 2, base, dims, strides, box, ones, CU_TENSOR_MAP_INTERLEAVE_NONE,
                CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   };
@@ -926,7 +929,7 @@ cudaError_t launch_ffn_tensor_core(const LaunchCtx &c, const TcMaps *maps, const
   const int ri = ru == 128 ? 0 : ru == 64 ? 1 : 2;
   TcArgs a;
   a.ru = ru;
-  a.ru_down = tc_rows_per_down_unit(ru);
+  a.ru_down = c.ru_down;
   a.kchunks_up = D.d / kChunkK;
   a.kchunks_down = D.f / kChunkK;
   const int n_pad_max = c.M >= kMaxTokChunk ? kMaxTokChunk : (c.M + kTokBox - 1) / kTokBox * kTokBox;

@@ -33,7 +33,7 @@ constexpr int kTokBox = 32;                // token rows per TMA box of the B op
 constexpr int kTokBoxSmall = 16;           // ... for units of at most 16 rows (the smallest MMA N)
 constexpr int kMaxTokChunk = 128;          // tokens per work unit: gate and up accumulators of two units fit TMEM
 
-// One tensor-core work unit: a slab of RU (128, 64 or 32) rows of one expert's weight
+// One work unit: a slab of RU (128, 64 or 32) rows of one expert's weight
 // matrix against one chunk (<= 128) of that expert's routed rows.
 struct __align__(16) Unit {
   int expert;
@@ -96,7 +96,8 @@ struct LaunchCtx {
   int M, k, B;
   int R_cap;            // max_M * max_k
   cudaStream_t stream;
-  int ru;               // weight rows per tensor-core work unit for this call (0: CUDA-core path)
+  int ru;               // weight rows per gate/up work unit for this call (0: routing only, no work units)
+  int ru_down = 0;      // ... per down unit
   int early = 0;        // 1: the FFN kernel starts on the shortlist before routing has finished (see ffn_tc.cu)
   int dense_all = 0;    // 1: every gate/up unit takes ALL tokens straight from `hidden` (trees of at most 16
                         //    tokens: the smallest MMA holds them anyway), so no gathered copy is made
@@ -141,11 +142,14 @@ cudaError_t launch_route_after_router(const LaunchCtx &c);           // route ke
 cudaError_t launch_calib_accumulate(const LaunchCtx &c);             // c_i += natural counts of the last router launch
 cudaError_t launch_gather(const LaunchCtx &c, const void *hidden);
 cudaError_t routing_configure();   // one-time function attributes of the routing kernels (tensor-core path)
-// ffn_simple.cu
-cudaError_t launch_ffn_cuda_core(const LaunchCtx &c, int phase);   // 0 gate/up, 1 down
+// ffn_cc.cu
+constexpr int kCcUnitCols = 32, kCcUnitDown = 64;   // f columns per gate/up unit, d columns per down unit
 cudaError_t cc_configure(const moespec_layer_desc &d, bool *fits);   // shared-memory opt-in of the CUDA-core FFN
+struct TcMaps;
+// both phases and the combine in one launch
+cudaError_t launch_ffn_cuda_core(const LaunchCtx &c, const TcMaps *maps, const void *hidden, void *out);
 // ffn_tc.cu
-struct TcMaps {            // per handle: weight maps for slab heights 128, 64, 32
+struct TcMaps {            // per handle: weight maps for boxes of 128, 64 and 32 rows of 128 bytes
   CUtensorMap w_gate[3], w_up[3], w_down[3];
   CUtensorMap x_perm[3], h_mid[3];   // token-row boxes of 32, 64 and 128 rows
   CUtensorMap x_perm16, h_mid16;     // ... and of 16 rows
@@ -170,8 +174,6 @@ cudaError_t tc_encode_maps(const moespec_layer_desc &d, const Workspace &ws, int
 cudaError_t tc_configure();   // one-time function attributes
 // gate/up + down + combine in one launch
 cudaError_t launch_ffn_tensor_core(const LaunchCtx &c, const TcMaps *maps, const void *hidden, void *out);
-// combine.cu
-cudaError_t launch_combine(const LaunchCtx &c, const void *hidden, void *out);
 // analysis.cu (oracle ranking of Eq. 6, reconstruction error of Section 4.5)
 constexpr int kSqdiffParts = 64;   // slices of the squared-difference reduction
 cudaError_t launch_gram(const LaunchCtx &c, double *gram, int *row2slot);

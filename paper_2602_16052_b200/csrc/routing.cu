@@ -489,7 +489,7 @@ struct RouteArgs {
   Workspace ws;
   int M, N, k, B;
   int policy, shortlist, renormalize;
-  int tiles_up, tiles_down;     // f/RU, d/RU slabs per expert (0 when the tensor-core path is not used)
+  int tiles_up, tiles_down;     // f/RU, d/RU slabs per expert (0: no work units are listed)
   long long expert_bytes;       // 3*d*f*sizeof(dtype)
   int early;                    // the FFN kernel starts on the shortlist before this kernel has finished
   int ffn_ctas;                 // CTAs of the FFN kernel: CTA c starts on gate/up unit c of the list
@@ -875,7 +875,7 @@ __global__ void __launch_bounds__(kRouteWarps * 32) route_kernel(RouteArgs a) {
       }
     }
   } else if (warp >= 4 && warp < 7) {
-    // tensor-core work units (expert, token chunk, 128-row slab): all gate/up units, then all down
+    // work units (expert, token chunk, 128-row slab): all gate/up units, then all down
     // units, each group ordered by (expert, chunk, slab); ready counters and the dispenser start at 0
     if (a.tiles_up > 0) {
       const int lt = tid - 128, nthr = 96;
@@ -958,7 +958,7 @@ static cudaError_t launch_route_kernel(const LaunchCtx &c, const float *logits) 
   a.M = c.M; a.N = D.n_experts; a.k = c.k; a.B = c.B;
   a.policy = D.policy; a.shortlist = D.shortlist; a.renormalize = D.renormalize;
   a.tiles_up = c.ru > 0 ? D.f / c.ru : 0;
-  a.tiles_down = c.ru > 0 ? D.d / tc_rows_per_down_unit(c.ru) : 0;
+  a.tiles_down = c.ru > 0 ? D.d / c.ru_down : 0;
   a.expert_bytes = 3LL * D.d * D.f * dtype_bytes(D.dtype);
   a.early = c.ru > 0 ? c.early : 0;
   a.ffn_ctas = tc_grid_size(D.device);
@@ -1117,6 +1117,9 @@ cudaError_t routing_configure() {
   set((const void *)router_mma_kernel<__half, 8>);
   set((const void *)router_mma_kernel<__nv_bfloat16, 16>);
   set((const void *)router_mma_kernel<__half, 16>);
+  set((const void *)router_topk_kernel<float, 2>);
+  set((const void *)router_topk_kernel<float, 4>);
+  set((const void *)router_topk_kernel<float, 8>);
   set((const void *)softmax_topk_kernel);
   set((const void *)route_kernel<1>);
   set((const void *)route_kernel<2>);

@@ -290,8 +290,7 @@ class Layer:
         return st.as_dict()
 
     KERNEL_NAMES_TC = ("router_topk", "route", "gather", "ffn")
-    KERNEL_NAMES_TC_SMALL = ("router_topk", "route", "ffn")      # trees of at most 16 tokens: no gathered copy
-    KERNEL_NAMES_CC = ("router_topk", "route", "gather", "ffn_gate_up", "ffn_down", "combine")
+    KERNEL_NAMES_TC_SMALL = ("router_topk", "route", "ffn")      # trees of at most 16 tokens, CUDA-core layers
 
     def debug_set_wait(self, limit_cycles: int, ready_bias: int):
         """Test hook: bound of the device-side waits and a ready-counter bias that makes them run out."""
@@ -306,7 +305,7 @@ class Layer:
         n = C.c_int(0)
         _check(lib().moespec_get_kernel_times(self._h, C.cast(ms, C.c_void_p), 8, C.cast(C.byref(n), C.c_void_p)),
                "moespec_get_kernel_times")
-        names = {3: self.KERNEL_NAMES_TC_SMALL, 4: self.KERNEL_NAMES_TC}.get(n.value, self.KERNEL_NAMES_CC)
+        names = self.KERNEL_NAMES_TC_SMALL if n.value == 3 else self.KERNEL_NAMES_TC
         return {names[i]: float(ms[i]) for i in range(min(n.value, len(names)))}
 
     def last_launch_count(self) -> int:

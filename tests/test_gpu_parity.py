@@ -130,6 +130,18 @@ def test_generator_is_bit_identical_on_gpu():
     assert torch.equal(wc, wg.cpu()) and torch.equal(bc, bg.cpu())
 
 
+# ------------------------------------------------------------------ CUDA-core FFN at the edges of its tiles
+@pytest.mark.parametrize("dtype", ["fp32", "bf16", "fp16"])
+def test_cuda_core_ffn_row_counts(dtype):
+    """Every split of a unit's rows over the threads (one to eight rows per thread, one, two and four row groups),
+    chunks of more than one pass and more than one chunk, at widths that are odd multiples of 64.  Tolerance: the
+    suite's bars, 1e-5 relative for fp32 and 2e-2 / 5e-3 of the RMS for 16-bit intermediates."""
+    cfg = synth.CONFIGS["tiny"].with_(d=192, f=320, n_experts=3, k=3, dtype=dtype)
+    for M in [1, 2, 3, 5, 8, 9, 15, 16, 17, 20, 25, 32, 33, 41, 49, 63, 64, 65, 97, 128, 129, 200, 300]:
+        _, _, st = run_e2e(cfg, M, 3, orc.SUBSTITUTION, orc.FROM_ALL, True, ms().FFN_CUDA_CORE, seed=M)
+        assert st["n_rows"] == 3 * M          # every expert has all M rows
+
+
 # ------------------------------------------------------------------ integer half, bit exact
 ROUTE_SHAPES = [
     ("tiny", dict(), [1, 15], [1, 2, 4, 8, 16, 40]),
