@@ -34,126 +34,204 @@ __device__ __forceinline__ double warp_sum(double v) {
 }
 
 // G[t][a][b] = (w_a y_a) . (w_b y_b) for the k slots of token t; slots without a row give zeros.
-// Grid M, 256 threads: the k(k+1)/2 pairs are dealt to the 8 warps, a warp walks the two rows together.
-__global__ void __launch_bounds__(256) gram_kernel(const float *__restrict__ y, const float *__restrict__ gate_w,
-                                                   const int *__restrict__ tokslot2row, double *__restrict__ gram,
-                                                   int *__restrict__ row2slot, int d, int k) {
+// One CTA per token.  What bounds it is the conversion of fp32 to fp64 (a product needs two, and they run at a
+// fraction of the FMA rate), so a warp takes row a against up to four rows b at a time: five conversions for four
+// products instead of eight, and the rows come from L1 after the first read.  Twelve warps are one round of k = 8.
+constexpr int kGramThreads = 384, kGramB = 4;
+
+__global__ void __launch_bounds__(kGramThreads) gram_kernel(const float *__restrict__ y, const float *__restrict__ gate_w,
+                                                            const int *__restrict__ tokslot2row,
+                                                            double *__restrict__ gram, int *__restrict__ row2slot,
+                                                            int d, int k) {
   const int t = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (threadIdx.x < k) {
     const int row = tokslot2row[(size_t)t * k + threadIdx.x];
     if (row >= 0) row2slot[row] = threadIdx.x;
   }
-  const int n_pairs = k * (k + 1) / 2;
-  for (int p = warp; p < n_pairs; p += 8) {
-    // pair index -> (a, b), a <= b
-    int a = 0, rem = p;
-    while (rem >= k - a) {
-      rem -= k - a;
-      ++a;
-    }
-    const int b = a + rem;
-    const int ra = tokslot2row[(size_t)t * k + a], rb = tokslot2row[(size_t)t * k + b];
-    double acc = 0.0;
-    if (ra >= 0 && rb >= 0) {
-      const float4 *pa = reinterpret_cast<const float4 *>(y + (size_t)ra * d);
-      const float4 *pb = reinterpret_cast<const float4 *>(y + (size_t)rb * d);
-      for (int c = lane; c < d / 4; c += 32) {
-        const float4 u = __ldcg(pa + c), v = __ldcg(pb + c);
-        acc += (double)u.x * (double)v.x;
-        acc += (double)u.y * (double)v.y;
-        acc += (double)u.z * (double)v.z;
-        acc += (double)u.w * (double)v.w;
+  int item = warp;                       // items: (a, group of b), a ascending, k - a rows b = a .. k - 1 in groups
+  for (int a = 0; a < k; ++a) {
+    const int groups = (k - a + kGramB - 1) / kGramB;
+    for (; item < groups; item += kGramThreads / 32) {
+      const int b0 = a + item * kGramB;
+      const int ra = tokslot2row[(size_t)t * k + a];
+      int rb[kGramB];
+      double acc[kGramB];
+      const float4 *pb[kGramB];
+      const float4 *pa = reinterpret_cast<const float4 *>(y + (size_t)max(ra, 0) * d);
+#pragma unroll
+      for (int q = 0; q < kGramB; ++q) {
+        acc[q] = 0.0;
+        rb[q] = b0 + q < k ? tokslot2row[(size_t)t * k + b0 + q] : -1;
+        pb[q] = rb[q] >= 0 ? reinterpret_cast<const float4 *>(y + (size_t)rb[q] * d) : pa;
       }
-      acc = warp_sum(acc);
-      acc *= (double)gate_w[(size_t)t * k + a] * (double)gate_w[(size_t)t * k + b];
+      if (ra >= 0)
+#pragma unroll 4
+        for (int c = lane; c < d / 4; c += 32) {
+          const float4 u = pa[c];
+          const double ux = (double)u.x, uy = (double)u.y, uz = (double)u.z, uw = (double)u.w;
+#pragma unroll
+          for (int q = 0; q < kGramB; ++q) {
+            const float4 v = pb[q][c];
+            acc[q] += ux * (double)v.x;
+            acc[q] += uy * (double)v.y;
+            acc[q] += uz * (double)v.z;
+            acc[q] += uw * (double)v.w;
+          }
+        }
+#pragma unroll
+      for (int q = 0; q < kGramB; ++q) {
+        const int b = b0 + q;
+        if (b >= k) break;                               // the same for the whole warp
+        double g = 0.0;
+        if (ra >= 0 && rb[q] >= 0)
+          g = warp_sum(acc[q]) * ((double)gate_w[(size_t)t * k + a] * (double)gate_w[(size_t)t * k + b]);
+        if (lane == 0) {
+          gram[((size_t)t * k + a) * k + b] = g;
+          gram[((size_t)t * k + b) * k + a] = g;
+        }
+      }
     }
-    if (lane == 0) {
-      gram[((size_t)t * k + a) * k + b] = acc;
-      gram[((size_t)t * k + b) * k + a] = acc;
-    }
+    item -= groups;
   }
 }
 
-// Greedy loop of Eq. 6 in one CTA of 256 threads.  Per step: warp w computes the gain of experts
-// w, w+8, ... (lanes stride the expert's rows in gather order, partial sums meet in a shuffle tree), then
-// warp 0 takes the largest gain (ties -> lower index; an expert without rows has gain 0).
-__global__ void __launch_bounds__(256) greedy_kernel(const double *__restrict__ gram, const int *__restrict__ assign_idx,
-                                                     const int *__restrict__ offset, const int *__restrict__ perm_row2tok,
-                                                     const int *__restrict__ row2slot, int M, int N, int k, int n_pick,
-                                                     int *__restrict__ order, double *__restrict__ objective,
-                                                     double *__restrict__ gold_energy) {
+// Greedy loop of Eq. 6 in one CTA.  gain(row) = 2 * sum of the row's Gram entries over the token's experts outside S,
+// minus its own: kept per routed row, so that a step recomputes only the rows of tokens that hold the expert just
+// picked (the same sum in the same order as from scratch) and otherwise adds up kept numbers.  Eight lanes take one
+// expert: they stride its rows in gather order and their partial sums meet in a shuffle tree, the same shape for every
+// expert, so identical experts tie exactly.  Every warp then finds the largest gain for itself (ties -> lower index; an
+// expert without rows has gain 0) by integer warp reductions of the order-preserving bit pattern.  What bounds a step is
+// its chain of dependent loads, additions and barriers, so everything it reads lies in shared memory where it fits (a
+// tree of 63 tokens with k = 8 needs 42 KB).  Ranking the first 32 of 64 experts at that size, layer pass included:
+// recomputing every row in every step 481 us; keeping row gains 266; eight-lane sums and integer maxima 235; shared
+// memory 229.
+constexpr int kGreedyThreads = 1024;
+
+__device__ __forceinline__ double row_gain(const double *gram, const int *assign_idx, int t, int a, int k,
+                                           const unsigned char *s_in, int also) {
+  const double *G = gram + ((size_t)t * k + a) * k;
+  const int *as = assign_idx + (size_t)t * k;
+  double cross = 0.0;
+  for (int b0 = 0; b0 < k; b0 += 8) {            // the loads of eight terms are in flight together
+    int j[8];
+    double g[8];
+#pragma unroll
+    for (int b = 0; b < 8; ++b) {
+      j[b] = b0 + b < k ? as[b0 + b] : -1;
+      g[b] = b0 + b < k ? G[b0 + b] : 0.0;
+    }
+#pragma unroll
+    for (int b = 0; b < 8; ++b)
+      if (j[b] >= 0 && j[b] != also && !s_in[j[b]]) cross += g[b];
+  }
+  return 2.0 * cross - G[a];
+}
+
+// larger double, larger key
+__device__ __forceinline__ unsigned long long order_bits(double v) {
+  if (v == 0.0) v = 0.0;                         // -0 and +0 share a key
+  const unsigned long long u = (unsigned long long)__double_as_longlong(v);
+  return (u >> 63) ? ~u : (u | 0x8000000000000000ull);
+}
+
+// Bytes of the working set: row gains, Gram matrices, kept experts, rows of the slots, tokens of the rows.
+size_t greedy_bytes(int M, int k) { return (size_t)M * k * (8 + 8 * (size_t)k + 4 + 4 + 4); }
+constexpr size_t kGreedySmem = 200 * 1024;
+
+// gain_mem: scratch, one double per routed row; used when the working set stays in global memory (in_smem = 0).
+__global__ void __launch_bounds__(kGreedyThreads) greedy_kernel(
+    const double *gram, const int *assign_idx, const int *__restrict__ offset, const int *perm_row2tok,
+    const int *tokslot2row, const int *__restrict__ row2slot, const int *__restrict__ status, double *gain_mem, int M,
+    int N, int k, int n_pick, int in_smem, RankingResult res) {
+  extern __shared__ double s_work[];
   __shared__ unsigned char s_in[kMaxExperts];
   __shared__ double s_gain[kMaxExperts];
-  __shared__ double s_part[8];
-  __shared__ double s_err;
-  __shared__ int s_best;
+  __shared__ int s_offset[kMaxExperts + 1];
+  __shared__ double s_part[kGreedyThreads / 32];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  for (int i = tid; i < N; i += blockDim.x) s_in[i] = 0;
+  for (int i = tid; i < N; i += kGreedyThreads) s_in[i] = 0;
+  for (int i = tid; i <= N; i += kGreedyThreads) s_offset[i] = offset[i];
+  double *gain = gain_mem;
+  const int pairs = M * k;
+  if (in_smem) {
+    gain = s_work;
+    double *sg = s_work + pairs;
+    int *sa = reinterpret_cast<int *>(sg + (size_t)pairs * k), *sr = sa + pairs, *sp = sr + pairs;
+    for (int i = tid; i < pairs * k; i += kGreedyThreads) sg[i] = gram[i];
+    const int R = offset[N];
+    for (int i = tid; i < pairs; i += kGreedyThreads) {
+      sa[i] = assign_idx[i];
+      sr[i] = tokslot2row[i];
+      sp[i] = i < R ? perm_row2tok[i] : 0;
+    }
+    gram = sg;
+    assign_idx = sa;
+    tokslot2row = sr;
+    perm_row2tok = sp;
+  }
+  __syncthreads();
   // objective of the empty set: sum_t || O*_t ||^2 = sum_t sum_{a,b} G_t[a][b], in a fixed order
+  double err = 0.0;
   {
     double acc = 0.0;
-    const size_t n = (size_t)M * k * k;
-    for (size_t i = tid; i < n; i += blockDim.x) acc += gram[i];
+    const size_t n = (size_t)pairs * k;
+    for (size_t i = tid; i < n; i += kGreedyThreads) acc += gram[i];
     acc = warp_sum(acc);
     if (lane == 0) s_part[warp] = acc;
     __syncthreads();
+    for (int w = 0; w < kGreedyThreads / 32; ++w) err += s_part[w];
     if (tid == 0) {
-      double tot = 0.0;
-      for (int w = 0; w < 8; ++w) tot += s_part[w];
-      s_err = tot;
-      *gold_energy = tot;
+      *res.gold = err;
+      *res.status = *status;
     }
   }
+  const int R = s_offset[N];
+  for (int r = tid; r < R; r += kGreedyThreads)
+    gain[r] = row_gain(gram, assign_idx, perm_row2tok[r], row2slot[r], k, s_in, -1);
   __syncthreads();
   for (int step = 0; step < n_pick; ++step) {
-    for (int i = warp; i < N; i += 8) {
+    for (int i0 = 0; i0 < N; i0 += kGreedyThreads / 8) {
+      const int i = i0 + (tid >> 3), sub = tid & 7;
       double g = 0.0;
-      if (!s_in[i]) {
-        for (int r = offset[i] + lane; r < offset[i + 1]; r += 32) {
-          const int t = perm_row2tok[r], a = row2slot[r];
-          const double *G = gram + ((size_t)t * k + a) * k;
-          double cross = 0.0;
-          for (int b = 0; b < k; ++b) {
-            const int j = assign_idx[(size_t)t * k + b];
-            if (j >= 0 && !s_in[j]) cross += G[b];
-          }
-          g += 2.0 * cross - G[a];
-        }
-        g = warp_sum(g);
-      }
-      if (lane == 0) s_gain[i] = g;
-    }
-    __syncthreads();
-    if (warp == 0) {
-      double best = 0.0;
-      int best_i = -1;
-      for (int i = lane; i < N; i += 32) {
-        if (s_in[i]) continue;
-        if (best_i < 0 || s_gain[i] > best) {        // ascending i: an equal gain keeps the lower index
-          best = s_gain[i];
-          best_i = i;
-        }
-      }
+      if (i < N && !s_in[i])
+        for (int r = s_offset[i] + sub; r < s_offset[i + 1]; r += 8) g += gain[r];
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        int lo = __double2loint(best), hi = __double2hiint(best);
+      for (int o = 4; o > 0; o >>= 1) {
+        int lo = __double2loint(g), hi = __double2hiint(g);
         lo = __shfl_xor_sync(kFullMask, lo, o);
         hi = __shfl_xor_sync(kFullMask, hi, o);
-        const double ob = __hiloint2double(hi, lo);
-        const int oi = __shfl_xor_sync(kFullMask, best_i, o);
-        if (oi >= 0 && (best_i < 0 || ob > best || (ob == best && oi < best_i))) {
-          best = ob;
-          best_i = oi;
-        }
+        g += __hiloint2double(hi, lo);
       }
-      if (lane == 0) {
-        s_best = best_i;
-        s_in[best_i] = 1;
-        s_err -= best;
-        order[step] = best_i;
-        objective[step] = s_err;
+      if (sub == 0 && i < N) s_gain[i] = g;
+    }
+    __syncthreads();
+    unsigned long long best = 0;
+    int best_i = 0x7fffffff;
+    for (int i = lane; i < N; i += 32) {
+      const unsigned long long key = order_bits(s_gain[i]);
+      if (!s_in[i] && (best_i == 0x7fffffff || key > best)) {      // ascending i: an equal gain keeps the lower index
+        best = key;
+        best_i = i;
       }
     }
+    const unsigned hi = __reduce_max_sync(kFullMask, (unsigned)(best >> 32));
+    const unsigned lo = __reduce_max_sync(kFullMask, (unsigned)(best >> 32) == hi ? (unsigned)best : 0u);
+    const bool mine = (unsigned)(best >> 32) == hi && (unsigned)best == lo;
+    best_i = (int)__reduce_min_sync(kFullMask, mine ? (unsigned)best_i : 0x7fffffffu);
+    err -= s_gain[best_i];
+    if (tid == 0) {
+      res.order[step] = best_i;
+      res.objective[step] = err;
+    }
+    // rows of the tokens that hold the expert just picked
+    const int first = s_offset[best_i], items = (s_offset[best_i + 1] - first) * k;
+    for (int q = tid; q < items; q += kGreedyThreads) {
+      const int t = perm_row2tok[first + q / k], a = q % k;
+      const int r = tokslot2row[(size_t)t * k + a];
+      if (r >= 0) gain[r] = row_gain(gram, assign_idx, t, a, k, s_in, best_i);
+    }
+    __syncthreads();
+    if (tid == 0) s_in[best_i] = 1;
     __syncthreads();
   }
 }
@@ -205,14 +283,19 @@ __global__ void sqdiff_final_kernel(const double *__restrict__ partial, int n_pa
 }  // namespace
 
 cudaError_t launch_gram(const LaunchCtx &c, double *gram, int *row2slot) {
-  gram_kernel<<<c.M, 256, 0, c.stream>>>(c.ws->y, c.ws->gate_w, c.ws->tokslot2row, gram, row2slot, c.desc->d, c.k);
+  gram_kernel<<<c.M, kGramThreads, 0, c.stream>>>(c.ws->y, c.ws->gate_w, c.ws->tokslot2row, gram, row2slot, c.desc->d, c.k);
   return cudaGetLastError();
 }
 
-cudaError_t launch_greedy(const LaunchCtx &c, const double *gram, const int *row2slot, int n_pick, int *order,
-                          double *objective, double *gold_energy) {
-  greedy_kernel<<<1, 256, 0, c.stream>>>(gram, c.ws->assign_idx, c.ws->offset, c.ws->perm_row2tok, row2slot, c.M,
-                                         c.desc->n_experts, c.k, n_pick, order, objective, gold_energy);
+cudaError_t launch_greedy(const LaunchCtx &c, const double *gram, const int *row2slot, int n_pick, double *row_gain,
+                          const RankingResult &res) {
+  const size_t bytes = greedy_bytes(c.M, c.k);
+  const bool in_smem = bytes <= kGreedySmem;
+  cudaError_t e = cudaFuncSetAttribute(greedy_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGreedySmem);
+  if (e != cudaSuccess) return e;
+  greedy_kernel<<<1, kGreedyThreads, in_smem ? bytes : 0, c.stream>>>(
+      gram, c.ws->assign_idx, c.ws->offset, c.ws->perm_row2tok, c.ws->tokslot2row, row2slot, c.ws->status, row_gain, c.M,
+      c.desc->n_experts, c.k, n_pick, in_smem, res);
   return cudaGetLastError();
 }
 

@@ -2,6 +2,7 @@
 #include "internal.h"
 
 #include <cstdlib>
+#include <cstring>
 #include <limits>
 #include <mutex>
 #include <new>
@@ -45,9 +46,10 @@ struct moespec_layer {
   int debug_ready_bias;
   unsigned epoch;       // bumped whenever something a captured graph has baked in changes
   // analysis mode (allocated by the first moespec_oracle_ranking / moespec_reconstruction_error call)
-  char *analysis;       // gram [max_M, max_k, max_k] f64 | row2slot [R_cap] | order [N] | objective [N] f64 | sums
-  double *an_gram, *an_objective, *an_sums, *an_partial;
-  int *an_row2slot, *an_order;
+  char *analysis;       // gram [max_M, max_k, max_k] f64 | row gains [R_cap] f64 | sums | row2slot [R_cap] | result
+  double *an_gram, *an_gain, *an_sums, *an_partial;
+  int *an_row2slot;
+  double *an_result;    // gold energy, objective [N] f64, then status, order [N] i32
   int an_M, an_k;       // shape of the Gram matrices held
 };
 
@@ -1068,6 +1070,9 @@ int moespec_stack_destroy(moespec_stack_t *S) {
 // ------------------------------------------------------------------ analysis mode
 namespace {
 
+// the ranking's result block: 1 + N doubles, then 1 + N ints
+size_t ranking_doubles(int N) { return (size_t)(1 + N) + (size_t)(2 + N) / 2; }
+
 int analysis_alloc(moespec_layer *L) {
   if (L->analysis) return MOESPEC_OK;
   const moespec_layer_desc &d = L->desc;
@@ -1076,11 +1081,11 @@ int analysis_alloc(moespec_layer *L) {
     c = Carver();
     c.base = base;
     c.take(L->an_gram, (size_t)d.max_M * d.max_k * d.max_k);
-    c.take(L->an_objective, (size_t)d.n_experts);
+    c.take(L->an_gain, (size_t)L->R_cap);
     c.take(L->an_sums, 4);
     c.take(L->an_partial, 2 * (size_t)kSqdiffParts);
     c.take(L->an_row2slot, (size_t)L->R_cap);
-    c.take(L->an_order, (size_t)d.n_experts);
+    c.take(L->an_result, ranking_doubles(d.n_experts));
     return (c.off + 255) & ~(size_t)255;
   };
   const size_t bytes = lay(nullptr);
@@ -1123,23 +1128,25 @@ int moespec_oracle_ranking(moespec_layer_t *L, const void *hidden, int M, int k,
   rc = run_layer(L, hidden, M, k, d.n_experts, dump, s, &full);
   if (rc) return rc;
   LaunchCtx c{&L->desc, &L->ws, M, k, d.n_experts, L->R_cap, s, 0};
+  const int N = d.n_experts;
+  int *ints = reinterpret_cast<int *>(L->an_result + 1 + N);
+  const RankingResult res{L->an_result, L->an_result + 1, ints, ints + 1};
   cudaError_t e = launch_gram(c, L->an_gram, L->an_row2slot);
   if (e == cudaSuccess)
-    e = launch_greedy(c, L->an_gram, L->an_row2slot, n_pick, L->an_order, L->an_objective, L->an_sums);
+    e = launch_greedy(c, L->an_gram, L->an_row2slot, n_pick, L->an_gain, res);
   if (e != cudaSuccess) return cuda_fail(e);
   L->an_M = M;
   L->an_k = k;
-  if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return cuda_fail(e);
-  if ((e = cudaMemcpy(order_host, L->an_order, sizeof(int) * n_pick, cudaMemcpyDeviceToHost)) != cudaSuccess)
-    return cuda_fail(e);
-  if (objective_host &&
-      (e = cudaMemcpy(objective_host, L->an_objective, sizeof(double) * n_pick, cudaMemcpyDeviceToHost)) != cudaSuccess)
-    return cuda_fail(e);
-  if (gold_energy_host &&
-      (e = cudaMemcpy(gold_energy_host, L->an_sums, sizeof(double), cudaMemcpyDeviceToHost)) != cudaSuccess)
-    return cuda_fail(e);
-  int status = 0;
-  if ((e = cudaMemcpy(&status, L->ws.status, sizeof(int), cudaMemcpyDeviceToHost)) != cudaSuccess) return cuda_fail(e);
+  // one copy: order, objective, gold energy and the status of the pass
+  double host[2 * (kMaxExperts + 2)];
+  e = cudaMemcpyAsync(host, L->an_result, ranking_doubles(N) * sizeof(double), cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  if (e != cudaSuccess) return cuda_fail(e);
+  const int *host_ints = reinterpret_cast<const int *>(host + 1 + N);
+  memcpy(order_host, host_ints + 1, sizeof(int) * n_pick);
+  if (objective_host) memcpy(objective_host, host + 1, sizeof(double) * n_pick);
+  if (gold_energy_host) *gold_energy_host = host[0];
+  const int status = host_ints[0];
   return status;      // 0, or the device-side status of the unbudgeted pass
 }
 

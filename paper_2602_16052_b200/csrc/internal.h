@@ -177,8 +177,15 @@ cudaError_t launch_ffn_tensor_core(const LaunchCtx &c, const TcMaps *maps, const
 // analysis.cu (oracle ranking of Eq. 6, reconstruction error of Section 4.5)
 constexpr int kSqdiffParts = 64;   // slices of the squared-difference reduction
 cudaError_t launch_gram(const LaunchCtx &c, double *gram, int *row2slot);
-cudaError_t launch_greedy(const LaunchCtx &c, const double *gram, const int *row2slot, int n_pick, int *order,
-                          double *objective, double *gold_energy);
+struct RankingResult {     // device; one block, so that one copy brings it to the host
+  double *gold;            // [1], then
+  double *objective;       // [N]
+  int *status;             // [1], the device status of the unpruned pass, then
+  int *order;              // [N]
+};
+// row_gain: scratch, one double per routed row
+cudaError_t launch_greedy(const LaunchCtx &c, const double *gram, const int *row2slot, int n_pick, double *row_gain,
+                          const RankingResult &res);
 cudaError_t launch_sqdiff(const void *a, const void *b, size_t n, int dtype, double *partial, double *out,
                           cudaStream_t stream);
 
