@@ -253,9 +253,15 @@ int run_layer(moespec_layer *L, const void *hidden, int M, int k, int B, void *o
   LaunchCtx c{desc, &L->ws, M, k, B > L->desc.n_experts ? L->desc.n_experts : B, L->R_cap, stream, 0};
   c.res_first = L->desc.resident_first;
   c.res_count = L->desc.resident_count;
+  bool pair = false;
   if (L->use_tc) {
-    c.ru = tc_rows_per_unit(L->desc, M, k, c.B);
-    c.ru_down = tc_rows_per_down_unit(c.ru);
+    pair = pair_takes(*desc, M, k, c.B);
+    c.ru = pair ? kPairTile : tc_rows_per_unit(L->desc, M, k, c.B);
+    c.ru_down = pair ? kPairTile : tc_rows_per_down_unit(c.ru);
+    if (pair) {
+      c.chunk = kPairChunk;
+      c.rank_order = 1;
+    }
     c.early = tc_early_start(*desc, M) ? 1 : 0;
     c.dense_all = tc_dense_all(*desc, M) ? 1 : 0;
     // The early units follow the shortlist's rank order.  Router-based ranks follow the tokens' own
@@ -288,7 +294,14 @@ int run_layer(moespec_layer *L, const void *hidden, int M, int k, int B, void *o
     if ((e = launch_gather(c, L->use_tc ? hidden : nullptr)) != cudaSuccess) return cuda_fail(e);
     if ((e = mark(++launches)) != cudaSuccess) return cuda_fail(e);
   }
-  if (L->use_tc) {
+  if (pair) {
+    for (int phase = 0; phase < 2; ++phase) {
+      if ((e = launch_ffn_pair(c, &L->maps, phase)) != cudaSuccess) return cuda_fail(e);
+      if ((e = mark(++launches)) != cudaSuccess) return cuda_fail(e);
+    }
+    if ((e = launch_combine(c, hidden, out)) != cudaSuccess) return cuda_fail(e);
+    if ((e = mark(++launches)) != cudaSuccess) return cuda_fail(e);
+  } else if (L->use_tc) {
     // both FFN phases and the combine are one persistent kernel
     if ((e = launch_ffn_tensor_core(c, &L->maps, hidden, out)) != cudaSuccess) return cuda_fail(e);
     if ((e = mark(++launches)) != cudaSuccess) return cuda_fail(e);
@@ -390,6 +403,7 @@ int moespec_layer_create(const moespec_layer_desc *desc, moespec_layer_t **out_l
     int cu_res = 0;
     e = tc_encode_maps(L->desc, L->ws, L->R_cap, &L->maps, &cu_res);
     if (e == cudaSuccess && use_tc) e = tc_configure();
+    if (e == cudaSuccess && use_tc) e = pair_configure();
     if (e == cudaSuccess) e = routing_configure();
     if (e != cudaSuccess) {
       cudaFree(L->arena);

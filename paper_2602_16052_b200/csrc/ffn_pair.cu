@@ -1,0 +1,566 @@
+// Tensor-core expert FFN for many tokens (bf16 and fp16): SM pairs.
+//
+// With a hundred and more rows per expert the FFN is bound by how fast an SM can feed its tensor core, not by HBM.  The
+// one-SM kernel (ffn_tc.cu) multiplies 128 weight rows by at most 128 token rows: such an MMA reads as many bytes of
+// shared memory as the SM can deliver while it runs, the incoming tiles compete with it, and every weight slab is
+// fetched once per 128 rows (2.6 GB of tiles for 16384 rows of the OLMoE shape: 472 us a layer).  Here two SMs work on
+// one tile with tcgen05.mma.cta_group::2: 256 weight rows (each SM holds 128 of them) times up to 256 token rows (each
+// SM holds half of them), so an SM reads 8 KB of shared memory and receives 1.5 KB (gate/up: the token rows serve two
+// matrices) or 2 KB (down) per 128 x 256 x 16 products, half of the above.
+//
+//   gate/up unit   256 f columns x (<= 256) rows: accumulators D_g, D_u, each n_pad columns in either SM's TMEM;
+//                  h_mid[row, col] = round(silu(D_g) * D_u)
+//   down unit      256 d columns x (<= 256) rows: y[row, col] = D (fp32)
+//
+// The two phases and the combine are launches of their own, so no unit waits for another.  Persistent: one CTA pair
+// per two SMs, units drawn in list order from a dispenser.
+//   warp 0     producer (both CTAs): this SM's weight rows and its half of the token rows, 64-element K slices, a
+//              ring of 4 (gate/up, 48 KB) or 3 (down, 64 KB: two slices) stages.  Both SMs' copies complete on the
+//              leader's barrier.
+//   warp 1     leader only: issues the MMAs of the pair; commits free the stage in both CTAs
+//   warp 2     leader only: draws units and hands them to both CTAs
+//   warps 4-19 epilogue of this SM's 128 weight rows (four warps per TMEM lane quarter, 16-column groups in turn)
+// TMEM is two slots of 256 columns.  A down unit, or a gate/up unit of at most 128 rows, takes one, so its epilogue
+// overlaps the next unit's MMAs; a larger gate/up unit takes both.
+// Every wait is bounded: on expiry the CTA raises its abort flag and records MOESPEC_ERR_TIMEOUT; the other CTA of
+// the pair runs into its own limit; copies are drained, both meet at a cluster barrier, free TMEM and return.
+#include "internal.h"
+
+namespace moespec {
+
+namespace {
+
+constexpr int kPEpiWarps = 16;
+constexpr int kPFirstEpi = 4;                         // a multiple of four: warp & 3 is the TMEM lane quarter
+constexpr int kPThreads = (kPFirstEpi + kPEpiWarps) * 32;
+constexpr int kPK = 64;                               // K elements per slice: one 128-byte swizzle row
+constexpr int kPTile = 16 * 1024;                     // 128 rows x 128 bytes
+constexpr int kPStageMem = 192 * 1024;
+constexpr int kPMaxStages = 4;
+constexpr int kPQueue = 2;                            // one unit in work, one drawn ahead
+constexpr int kPSmem = kPStageMem + 1024 + 1024;
+constexpr long long kPSpinCycles = 2000000000LL;      // default bound of every wait: ~1 s at 2 GHz
+
+struct PairMaps {
+  CUtensorMap w[2];          // gate and up, or down and unused: boxes of 128 rows
+  CUtensorMap rows[3];       // x_perm or h_mid: boxes of 32, 64, 128 rows
+};
+
+struct PairArgs {
+  const Unit *units;
+  const int *n_units;        // [0] gate/up units, [1] down units
+  int *dispenser;            // of this phase; zeroed by the router kernel of the call
+  const int *ready;          // test hook: with hold > 0 the down phase waits for ready[0] to reach it (it never does)
+  int hold;
+  int phase;
+  int cps;                   // K slices per stage
+  int k_iters;               // stages per unit: K / 64 / cps
+  int n_stages, stage_bytes;
+  void *h_mid;               // [R, f]
+  float *y;                  // [R, d]
+  int f, d, is_fp16;
+  int res_first;
+  int *status;
+  long long spin_limit;
+};
+
+__device__ __forceinline__ uint32_t p_smem(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ uint32_t p_map(uint32_t addr, uint32_t rank) {      // the same place in CTA `rank` of the pair
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void p_bar_init(uint32_t bar, uint32_t count) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
+}
+// Arrival at a barrier of either CTA.  publish: this thread's earlier stores to the other CTA's shared memory are
+// visible to whoever waits there with p_bar_wait<true>; the plain forms order shared and tensor memory only within a
+// CTA, which is all the other barriers need (copies and MMAs order their own data).  Cluster-scope acquires in every
+// wait cost 30 us of 380 at 2048 tokens.
+__device__ __forceinline__ void p_arrive(uint32_t mapped_bar) {
+  asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(mapped_bar) : "memory");
+}
+__device__ __forceinline__ void p_arrive_publish(uint32_t mapped_bar) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(mapped_bar) : "memory");
+}
+__device__ __forceinline__ void p_expect_tx(uint32_t bar, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
+template <bool kPublished = false>
+__device__ __forceinline__ bool p_bar_try(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  if constexpr (kPublished)
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+  else
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+  return ok != 0;
+}
+// Bounded wait.  Returns false when the CTA is aborting or the limit expired.
+template <bool kPublished = false>
+__device__ __forceinline__ bool p_bar_wait(uint32_t bar, uint32_t parity, volatile int *abort_flag, long long limit) {
+  if (p_bar_try<kPublished>(bar, parity)) return true;
+  const long long t0 = clock64();
+  for (uint32_t i = 1;; ++i) {
+    if (p_bar_try<kPublished>(bar, parity)) return true;
+    if ((i & 255u) == 0u) {
+      if (*abort_flag) return false;
+      if (clock64() - t0 > limit) {
+        *abort_flag = 1;
+        return false;
+      }
+    }
+  }
+}
+__device__ __forceinline__ void p_cluster_sync() {
+  asm volatile("barrier.cluster.arrive.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+}
+// Copies into this CTA's shared memory that complete on the leader's barrier.
+__device__ __forceinline__ void p_load_w(uint32_t dst, const CUtensorMap *map, uint32_t leader_bar, int c0, int c1, int c2) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
+      ::"r"(dst), "l"(map), "r"(leader_bar), "r"(c0), "r"(c1), "r"(c2)
+      : "memory");
+}
+__device__ __forceinline__ void p_load_rows(uint32_t dst, const CUtensorMap *map, uint32_t leader_bar, int c0, int c1) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
+      ::"r"(dst), "l"(map), "r"(leader_bar), "r"(c0), "r"(c1)
+      : "memory");
+}
+__device__ __forceinline__ void p_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void p_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
+// Arrives on the barrier at this offset in both CTAs once the MMAs issued so far have completed.
+__device__ __forceinline__ void p_commit(uint32_t bar) {
+  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
+               "h"((uint16_t)3)
+               : "memory");
+}
+__device__ __forceinline__ void p_mma(uint32_t tmem_d, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+      ::"r"(tmem_d), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+__device__ __forceinline__ void p_ld16(uint32_t taddr, uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr)
+      : "memory");
+}
+__device__ __forceinline__ void p_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+
+// K-major operand, 128-byte swizzle, rows at a 128-byte pitch, groups of eight rows 1024 bytes apart.
+__device__ __forceinline__ uint64_t p_desc(uint32_t addr) {
+  return (uint64_t)((addr & 0x3FFFFu) >> 4) | ((uint64_t)1 << 16) | ((uint64_t)(1024 >> 4) << 32) | ((uint64_t)1 << 46) |
+         ((uint64_t)2 << 61);
+}
+
+// Which TMEM slots a unit takes, followed in the same way by the MMA issuer and the epilogue warps of both CTAs:
+// full[] / empty[] count the uses of the two slots' barriers.
+struct SlotState {
+  uint32_t next = 0, full[2] = {0, 0}, empty[2] = {0, 0};
+};
+
+// rows of a unit on the MMA's N axis: either SM holds half of them, and copies come in boxes of 32
+__device__ __forceinline__ int pair_pad(int n_rows) { return (n_rows + 63) & ~63; }
+
+__global__ void __launch_bounds__(kPThreads, 1) __cluster_dims__(2, 1, 1)
+    ffn_pair_kernel(const __grid_constant__ PairMaps maps, PairArgs a) {
+  extern __shared__ __align__(1024) uint8_t p_smem_raw[];
+  const uint32_t base = (p_smem(p_smem_raw) + 1023u) & ~1023u;      // the same offset in both CTAs
+  uint8_t *ctrl_gen = p_smem_raw + (base - p_smem(p_smem_raw)) + kPStageMem;
+  const uint32_t ctrl = base + kPStageMem;
+  const uint32_t bar_full = ctrl, bar_empty = ctrl + 8 * kPMaxStages;
+  const uint32_t bar_acc_full = ctrl + 16 * kPMaxStages, bar_acc_empty = bar_acc_full + 16;      // [2] each
+  const uint32_t bar_q_full = bar_acc_empty + 16, bar_q_empty = bar_q_full + 8 * kPQueue;
+  volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(ctrl_gen + 240);
+  volatile int *abort_flag = reinterpret_cast<volatile int *>(ctrl_gen + 244);
+  constexpr uint32_t kQOff = 256;
+  Unit *queue = reinterpret_cast<Unit *>(ctrl_gen + kQOff);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  uint32_t rank;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+  const bool leader = rank == 0;
+
+  pdl_trigger();
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kPMaxStages; ++s) {
+      p_bar_init(bar_full + 8 * s, 1);
+      p_bar_init(bar_empty + 8 * s, 1);
+    }
+    for (int b = 0; b < 2; ++b) {
+      p_bar_init(bar_acc_full + 8 * b, 1);
+      p_bar_init(bar_acc_empty + 8 * b, 2 * kPEpiWarps);
+    }
+    for (int q = 0; q < kPQueue; ++q) {
+      p_bar_init(bar_q_full + 8 * q, 1);
+      p_bar_init(bar_q_empty + 8 * q, 2 * kPEpiWarps + 3);      // epilogue warps, the MMA issuer, the producers
+    }
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(
+                     p_smem(const_cast<uint32_t *>(tmem_slot)))
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+  }
+  p_fence_before();
+  __syncthreads();
+  p_cluster_sync();            // the barriers of both CTAs exist
+  p_fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+  pdl_wait();
+
+  const int first_unit = a.phase == 0 ? 0 : a.n_units[0];
+  const int n_units = a.phase == 0 ? a.n_units[0] : a.n_units[1];
+  const uint32_t w_tiles = a.phase == 0 ? 2 : (uint32_t)a.cps;      // weight tiles of a stage (gate/up: one slice of each)
+
+  if (warp == 0) {
+    if (lane == 0) {
+      // ----------------------------------------------------------------- producer
+      uint32_t it = 0, s = 0, ph = 0;      // stages used so far; slot of the ring and its parity
+      bool ok = true;
+      for (uint32_t qi = 0; ok; ++qi) {
+        const uint32_t q = qi % kPQueue, qph = (qi / kPQueue) & 1u;
+        if (!p_bar_wait<true>(bar_q_full + 8 * q, qph, abort_flag, a.spin_limit)) { ok = false; break; }
+        const int expert = queue[q].expert - a.res_first, tile = queue[q].tile, u_row0 = queue[q].row0,
+                  n_rows = queue[q].n_rows;
+        const bool end = queue[q].expert < 0;
+        p_arrive(p_map(bar_q_empty + 8 * q, 0));
+        if (end) break;
+        const int half = pair_pad(n_rows) / 2;
+        const int bsel = half == 128 ? 2 : half == 64 ? 1 : 0, box = 32 << bsel;
+        const uint32_t bytes = w_tiles * kPTile + (uint32_t)(a.cps * half) * 128u;
+        const int w_row = tile * 256 + (int)rank * 128, row0 = u_row0 + (int)rank * half;
+        for (int kc = 0; kc < a.k_iters; ++kc, ++it) {
+          if (!p_bar_wait(bar_empty + 8 * s, ph ^ 1u, abort_flag, a.spin_limit)) { ok = false; break; }
+          const uint32_t stage = base + s * (uint32_t)a.stage_bytes, full = p_map(bar_full + 8 * s, 0);
+          if (leader) p_expect_tx(bar_full + 8 * s, 2 * bytes);
+          for (int j = 0; j < a.cps; ++j) {
+            const int col = (kc * a.cps + j) * kPK;
+            p_load_w(stage + j * kPTile, &maps.w[0], full, col, w_row, expert);
+            if (a.phase == 0) p_load_w(stage + kPTile, &maps.w[1], full, col, w_row, expert);
+            for (int r = 0; r < half; r += box)
+              p_load_rows(stage + (w_tiles + j) * kPTile + r * 128, &maps.rows[bsel], full, col, row0 + r);
+          }
+          if (++s == (uint32_t)a.n_stages) { s = 0; ph ^= 1u; }
+        }
+      }
+      const uint32_t lo = it > (uint32_t)a.n_stages ? it - a.n_stages : 0u;
+      if (ok) {                 // the commits that free the last stages have arrived here before this CTA leaves
+        for (uint32_t j = lo; j < it && ok; ++j)
+          ok = p_bar_wait(bar_empty + 8 * (j % a.n_stages), (j / a.n_stages) & 1u, abort_flag, a.spin_limit);
+      }
+      if (!ok && leader) {      // giving up: what is on its way into either CTA lands first (bounded)
+        for (uint32_t j = lo; j < it; ++j) {
+          const long long t0 = clock64();
+          while (!p_bar_try(bar_full + 8 * (j % a.n_stages), (j / a.n_stages) & 1u))
+            if (clock64() - t0 > a.spin_limit) break;
+        }
+      }
+    }
+    __syncwarp();
+  } else if (warp == 1) {
+    if (leader && lane == 0) {
+      // ----------------------------------------------------------------- MMA issuer of the pair
+      uint32_t s = 0, ph = 0;
+      SlotState sl;
+      bool ok = true;
+      const uint32_t fmt = a.is_fp16 ? 0u : 1u;
+      for (uint32_t qi = 0; ok; ++qi) {
+        const uint32_t q = qi % kPQueue, qph = (qi / kPQueue) & 1u;
+        if (!p_bar_wait<true>(bar_q_full + 8 * q, qph, abort_flag, a.spin_limit)) break;
+        const int expert = queue[q].expert, n_rows = queue[q].n_rows;
+        p_arrive(p_map(bar_q_empty + 8 * q, 0));
+        if (expert < 0) break;
+        const int n_pad = pair_pad(n_rows);
+        const uint32_t idesc = (1u << 4) | (fmt << 7) | (fmt << 10) | ((uint32_t)(n_pad >> 3) << 17) | (16u << 24);
+        const bool both = a.phase == 0 && n_pad > 128;
+        const uint32_t slot = both ? 0u : sl.next;
+        ok = p_bar_wait(bar_acc_empty + 8 * slot, (sl.empty[slot] & 1u) ^ 1u, abort_flag, a.spin_limit);
+        if (ok && both) ok = p_bar_wait(bar_acc_empty + 8, (sl.empty[1] & 1u) ^ 1u, abort_flag, a.spin_limit);
+        if (!ok) break;
+        ++sl.empty[slot];
+        if (both) ++sl.empty[1];
+        sl.next = both ? 0u : slot ^ 1u;
+        p_fence_after();
+        const uint32_t tmem_d = tmem_base + slot * 256u, tmem_u = tmem_d + (uint32_t)(both ? 256 : n_pad);
+        for (int kc = 0; kc < a.k_iters; ++kc) {
+          if (!p_bar_wait(bar_full + 8 * s, ph, abort_flag, a.spin_limit)) { ok = false; break; }
+          p_fence_after();
+          uint64_t ad = p_desc(base + s * (uint32_t)a.stage_bytes), bd = ad + w_tiles * (kPTile >> 4);
+          if (a.phase == 0) {
+#pragma unroll
+            for (int kk = 0; kk < kPK / 16; ++kk) {
+              const uint32_t acc = kc > 0 || kk > 0;
+              p_mma(tmem_d, ad + 2 * kk, bd + 2 * kk, idesc, acc);
+              p_mma(tmem_u, ad + (kPTile >> 4) + 2 * kk, bd + 2 * kk, idesc, acc);
+            }
+          } else {
+            for (int j = 0; j < a.cps; ++j, ad += kPTile >> 4, bd += kPTile >> 4)
+#pragma unroll
+              for (int kk = 0; kk < kPK / 16; ++kk)
+                p_mma(tmem_d, ad + 2 * kk, bd + 2 * kk, idesc, kc > 0 || j > 0 || kk > 0);
+          }
+          p_commit(bar_empty + 8 * s);       // both CTAs may refill the stage
+          if (++s == (uint32_t)a.n_stages) { s = 0; ph ^= 1u; }
+        }
+        if (!ok) break;
+        p_commit(bar_acc_full + 8 * slot);
+      }
+    }
+    __syncwarp();
+  } else if (warp == 2) {
+    if (leader && lane == 0) {
+      // ----------------------------------------------------------------- scheduler of the pair
+      // Draws units in list order and hands them to both CTAs.  A thread of its own: ticket, list entry and the
+      // publication to the other CTA are three round trips, which stood between two units when the producer made them
+      // (2048 tokens, OLMoE shape: 378 us a layer; hidden 363; hidden, with two K slices per down stage, 348).
+      bool ok = true;
+      if (a.hold > 0) {
+        const long long t0 = clock64();
+        while (*reinterpret_cast<const volatile int *>(a.ready) < a.hold) {
+          if (clock64() - t0 > a.spin_limit) { *abort_flag = 1; ok = false; break; }
+          __nanosleep(128);
+        }
+      }
+      for (uint32_t qi = 0; ok; ++qi) {
+        const uint32_t q = qi % kPQueue, qph = (qi / kPQueue) & 1u;
+        if (!p_bar_wait(bar_q_empty + 8 * q, qph ^ 1u, abort_flag, a.spin_limit)) break;
+        Unit un{};
+        un.expert = -1;
+        const int ticket = atomicAdd(a.dispenser, 1);
+        if (ticket < n_units) un = a.units[first_unit + ticket];
+        queue[q] = un;
+        const uint32_t other = p_map(ctrl + kQOff + q * (uint32_t)sizeof(Unit), 1);
+        asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(other), "r"(un.expert), "r"(un.tile),
+                     "r"(un.row0), "r"(un.n_rows)
+                     : "memory");
+        p_arrive_publish(p_map(bar_q_full + 8 * q, 1));
+        p_arrive_publish(p_map(bar_q_full + 8 * q, 0));
+        if (un.expert < 0) break;
+      }
+    }
+    __syncwarp();
+  } else if (warp >= kPFirstEpi) {
+    // ------------------------------------------------------------------- epilogue
+    const int quarter = warp & 3;
+    constexpr int kEpiStep = 16 * kPEpiWarps / 4;
+    const int c_first = ((warp - kPFirstEpi) >> 2) * 16;
+    const uint32_t lane_off = (uint32_t)(quarter * 32) << 16;
+    SlotState sl;
+    for (uint32_t qi = 0;; ++qi) {
+      const uint32_t q = qi % kPQueue, qph = (qi / kPQueue) & 1u;
+      if (!p_bar_wait<true>(bar_q_full + 8 * q, qph, abort_flag, a.spin_limit)) break;
+      const int expert = queue[q].expert, tile = queue[q].tile, row0 = queue[q].row0, n_rows = queue[q].n_rows;
+      __syncwarp();
+      if (lane == 0) p_arrive(p_map(bar_q_empty + 8 * q, 0));
+      if (expert < 0) break;
+      const int n_pad = pair_pad(n_rows);
+      const bool both = a.phase == 0 && n_pad > 128;
+      const uint32_t slot = both ? 0u : sl.next;
+      sl.next = both ? 0u : slot ^ 1u;
+      if (!p_bar_wait(bar_acc_full + 8 * slot, sl.full[slot] & 1u, abort_flag, a.spin_limit)) break;
+      ++sl.full[slot];
+      __syncwarp();
+      p_fence_after();
+      const uint32_t taddr = tmem_base + lane_off + slot * 256u, taddr_u = taddr + (uint32_t)(both ? 256 : n_pad);
+      const int col = tile * 256 + (int)rank * 128 + quarter * 32 + lane;       // along f or d
+      if (a.phase == 0) {
+        uint32_t g[16], up[16];               // the next group's accumulators are on their way while this one is stored
+        if (c_first < n_rows) {
+          p_ld16(taddr + c_first, g);
+          p_ld16(taddr_u + c_first, up);
+        }
+        for (int c0 = c_first; c0 < n_rows; c0 += kEpiStep) {
+          p_ld_wait();
+          float m[16];
+#pragma unroll
+          for (int i = 0; i < 16; ++i) {
+            const float gv = __uint_as_float(g[i]);
+            m[i] = __fdividef(gv, 1.f + __expf(-gv)) * __uint_as_float(up[i]);
+          }
+          if (c0 + kEpiStep < n_rows) {
+            p_ld16(taddr + c0 + kEpiStep, g);
+            p_ld16(taddr_u + c0 + kEpiStep, up);
+          }
+          const int n_here = min(16, n_rows - c0);
+          if (a.is_fp16) {
+            __half *dst = reinterpret_cast<__half *>(a.h_mid) + (size_t)(row0 + c0) * a.f + col;
+#pragma unroll
+            for (int i = 0; i < 16; ++i)
+              if (i < n_here) dst[(size_t)i * a.f] = __float2half_rn(m[i]);
+          } else {
+            __nv_bfloat16 *dst = reinterpret_cast<__nv_bfloat16 *>(a.h_mid) + (size_t)(row0 + c0) * a.f + col;
+#pragma unroll
+            for (int i = 0; i < 16; ++i)
+              if (i < n_here) dst[(size_t)i * a.f] = __float2bfloat16_rn(m[i]);
+          }
+        }
+      } else {
+        for (int c0 = c_first; c0 < n_rows; c0 += kEpiStep) {
+          uint32_t g[16];
+          p_ld16(taddr + c0, g);
+          p_ld_wait();
+          const int n_here = min(16, n_rows - c0);
+          float *dst = a.y + (size_t)(row0 + c0) * a.d + col;
+#pragma unroll
+          for (int i = 0; i < 16; ++i)
+            if (i < n_here) dst[(size_t)i * a.d] = __uint_as_float(g[i]);
+        }
+      }
+      p_fence_before();
+      __syncwarp();
+      if (lane == 0) {
+        p_arrive(p_map(bar_acc_empty + 8 * slot, 0));
+        if (both) p_arrive(p_map(bar_acc_empty + 8, 0));
+      }
+    }
+  }
+
+  p_fence_before();
+  __syncthreads();
+  if (threadIdx.x == 0 && *abort_flag) atomicExch(a.status, (int)MOESPEC_ERR_TIMEOUT);
+  p_cluster_sync();            // neither CTA leaves, or frees TMEM, while the other may still use it
+  if (warp == 1) {
+    p_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, 512;" ::"r"(tmem_base) : "memory");
+  }
+}
+
+// out_t = sum over the kept slots of wgt[t, slot] * y[row(t, slot)], slots in a fixed order (outer sums of Eq. 2 / 7 /
+// 8), exact zeros for a token with no kept expert (Section 3.3).  Grid (M, d / 1024): four columns per thread, all of
+// up to eight rows loaded before the first FMA.
+template <typename T, typename TO>
+__global__ void __launch_bounds__(256) pair_combine_kernel(const float *__restrict__ y, const float *__restrict__ gate_w,
+                                                           const int *__restrict__ tokslot2row,
+                                                           const int *__restrict__ assign_idx,
+                                                           const T *__restrict__ hidden, TO *__restrict__ out, int d,
+                                                           int k, int residual, int res_first, int res_count) {
+  const int t = blockIdx.x, c = (blockIdx.y * 256 + threadIdx.x) * 4;
+  __shared__ int s_row[kMaxK];
+  __shared__ float s_w[kMaxK];
+  pdl_trigger();
+  pdl_wait();
+  if (threadIdx.x < k) {
+    int row = tokslot2row[(size_t)t * k + threadIdx.x];
+    if (res_count > 0 && row >= 0) {      // expert-parallel shard: only the slots of resident experts
+      const int e = assign_idx[(size_t)t * k + threadIdx.x];
+      if (e < res_first || e >= res_first + res_count) row = -1;
+    }
+    s_row[threadIdx.x] = row;
+    s_w[threadIdx.x] = gate_w[(size_t)t * k + threadIdx.x];
+  }
+  __syncthreads();
+  if (c >= d) return;
+  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int s0 = 0; s0 < k; s0 += 8) {
+    float4 v[8];
+#pragma unroll
+    for (int s = 0; s < 8; ++s) {
+      const int row = s0 + s < k ? s_row[s0 + s] : -1;
+      v[s] = row >= 0 ? __ldcs(reinterpret_cast<const float4 *>(y + (size_t)row * d + c)) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+#pragma unroll
+    for (int s = 0; s < 8; ++s)
+      if (s0 + s < k && s_row[s0 + s] >= 0) {
+        const float w = s_w[s0 + s];
+        acc.x = fmaf(w, v[s].x, acc.x);
+        acc.y = fmaf(w, v[s].y, acc.y);
+        acc.z = fmaf(w, v[s].z, acc.z);
+        acc.w = fmaf(w, v[s].w, acc.w);
+      }
+  }
+  if (residual) {
+    const T *h = hidden + (size_t)t * d + c;
+    acc.x += (float)h[0]; acc.y += (float)h[1]; acc.z += (float)h[2]; acc.w += (float)h[3];
+  }
+  if constexpr (sizeof(TO) == 4) {
+    *reinterpret_cast<float4 *>(out + (size_t)t * d + c) = acc;
+  } else {
+    alignas(8) TO o[4] = {(TO)acc.x, (TO)acc.y, (TO)acc.z, (TO)acc.w};
+    *reinterpret_cast<uint2 *>(out + (size_t)t * d + c) = *reinterpret_cast<const uint2 *>(o);
+  }
+}
+
+template <typename T, typename TO>
+cudaError_t launch_pair_combine(const LaunchCtx &c, const void *hidden, void *out) {
+  const moespec_layer_desc &D = *c.desc;
+  return launch_kernel(pair_combine_kernel<T, TO>, dim3(c.M, (D.d + 1023) / 1024), dim3(256), 0, c.stream,
+                       (const float *)c.ws->y, (const float *)c.ws->gate_w, (const int *)c.ws->tokslot2row,
+                       (const int *)c.ws->assign_idx, (const T *)hidden, (TO *)out, D.d, c.k, D.residual, c.res_first,
+                       c.res_count > 0 && c.res_count < D.n_experts ? c.res_count : 0);
+}
+
+}  // namespace
+
+cudaError_t pair_configure() {
+  return cudaFuncSetAttribute(ffn_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kPSmem);
+}
+
+// Whole pair tiles, and enough rows per kept expert.  The line lies where the two were measured equal (us a layer, one
+// SM / pairs, OLMoE shape): 300 tokens B=32 (75 rows per expert) 118 / 122, 512 tokens B=64 (64 rows) 203 / 218, 511
+// tokens B=32 (128 rows) 146 / 133, 1024 tokens B=64 (128 rows) 287 / 246, 2048 tokens B=64 (256 rows) 472 / 348.
+bool pair_takes(const moespec_layer_desc &D, int M, int k, int B) {
+  const int active = B < D.n_experts ? B : D.n_experts;
+  if (D.f % kPairTile || D.d % kPairTile) return false;
+  return M > 2 * kMaxTokChunk && (long long)M * k >= 96LL * active;
+}
+
+cudaError_t launch_ffn_pair(const LaunchCtx &c, const TcMaps *maps, int phase) {
+  const moespec_layer_desc &D = *c.desc;
+  const Workspace &ws = *c.ws;
+  PairMaps m;
+  m.w[0] = phase == 0 ? maps->w_gate[0] : maps->w_down[0];
+  m.w[1] = phase == 0 ? maps->w_up[0] : maps->w_down[0];
+  for (int i = 0; i < 3; ++i) m.rows[i] = phase == 0 ? maps->x_perm[i] : maps->h_mid[i];
+  PairArgs a;
+  a.units = ws.units;
+  a.n_units = ws.counters + 3;
+  a.dispenser = ws.unit_counter + (phase == 0 ? 0 : 2);
+  a.ready = ws.ready;
+  a.hold = phase == 0 ? 0 : c.debug_ready_bias;
+  a.phase = phase;
+  a.cps = phase == 0 ? 1 : 2;
+  a.k_iters = (phase == 0 ? D.d : D.f) / kPK / a.cps;
+  a.n_stages = phase == 0 ? 4 : 3;
+  a.stage_bytes = phase == 0 ? 3 * kPTile : 4 * kPTile;
+  a.h_mid = ws.h_mid;
+  a.y = ws.y;
+  a.f = D.f;
+  a.d = D.d;
+  a.is_fp16 = D.dtype == MOESPEC_FP16;
+  a.res_first = c.res_first;
+  a.status = ws.status;
+  a.spin_limit = c.debug_spin_limit > 0 ? c.debug_spin_limit : kPSpinCycles;
+  return launch_kernel(ffn_pair_kernel, dim3(tc_grid_size(D.device) & ~1), dim3(kPThreads), kPSmem, c.stream, m, a);
+}
+
+cudaError_t launch_combine(const LaunchCtx &c, const void *hidden, void *out) {
+  const moespec_layer_desc &D = *c.desc;
+  const bool same = D.out_dtype == 0 || D.out_dtype == D.dtype;
+  if (D.dtype == MOESPEC_BF16)
+    return same ? launch_pair_combine<__nv_bfloat16, __nv_bfloat16>(c, hidden, out)
+                : launch_pair_combine<__nv_bfloat16, float>(c, hidden, out);
+  return same ? launch_pair_combine<__half, __half>(c, hidden, out) : launch_pair_combine<__half, float>(c, hidden, out);
+}
+
+}  // namespace moespec

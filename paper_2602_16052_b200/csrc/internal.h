@@ -39,7 +39,7 @@ struct __align__(16) Unit {
   int expert;
   int tile;       // slab index along f (gate/up phase) or d (down phase)
   int row0;       // first routed row of the chunk
-  int n_rows;     // rows in the chunk (1..256)
+  int n_rows;     // rows in the chunk (1..128, or 256 for SM pairs)
   int chunk;      // global index of the (expert, token chunk) pair: indexes the ready counters
   int phase;      // 0 gate/up, 1 down
   int pad0, pad1;
@@ -79,7 +79,8 @@ struct Workspace {
   int *static_order;        // [N] the fixed ordering itself: expert at position r (first n_static entries)
   Unit *units;          // gate/up units (expert, chunk, tile ascending) followed by the down units
   int *ready;           // [chunks] gate/up units finished per (expert, token chunk); zeroed by the route kernel
-  int *unit_counter;    // [0] next unit to hand out, [1] finished down units; zeroed by the router kernel
+  int *unit_counter;    // [0] next unit to hand out, [1] finished down units, [2] next down unit (SM pairs); zeroed by
+                        // the router kernel
   int *counters;        // [0]=n_S [1]=n_active [2]=R [3]=n_units_up [4]=n_units_down
   moespec_stats *stats; // device copy
   int *status;          // device status word (0 = ok)
@@ -98,6 +99,8 @@ struct LaunchCtx {
   cudaStream_t stream;
   int ru;               // weight rows per gate/up work unit for this call (0: routing only, no work units)
   int ru_down = 0;      // ... per down unit
+  int chunk = kMaxTokChunk;   // most token rows per work unit
+  int rank_order = 0;   // 1: the unit list follows the shortlist's rank order also for many tokens
   int early = 0;        // 1: the FFN kernel starts on the shortlist before routing has finished (see ffn_tc.cu)
   int dense_all = 0;    // 1: every gate/up unit takes ALL tokens straight from `hidden` (trees of at most 16
                         //    tokens: the smallest MMA holds them anyway), so no gathered copy is made
@@ -174,6 +177,12 @@ cudaError_t tc_encode_maps(const moespec_layer_desc &d, const Workspace &ws, int
 cudaError_t tc_configure();   // one-time function attributes
 // gate/up + down + combine in one launch
 cudaError_t launch_ffn_tensor_core(const LaunchCtx &c, const TcMaps *maps, const void *hidden, void *out);
+// ffn_pair.cu
+constexpr int kPairTile = 256, kPairChunk = 256;      // weight rows and most token rows of a unit
+cudaError_t pair_configure();
+bool pair_takes(const moespec_layer_desc &d, int M, int k, int B);        // is a call left to the pair kernels?
+cudaError_t launch_ffn_pair(const LaunchCtx &c, const TcMaps *maps, int phase);      // 0 gate/up, 1 down
+cudaError_t launch_combine(const LaunchCtx &c, const void *hidden, void *out);
 // analysis.cu (oracle ranking of Eq. 6, reconstruction error of Section 4.5)
 constexpr int kSqdiffParts = 64;   // slices of the squared-difference reduction
 cudaError_t launch_gram(const LaunchCtx &c, double *gram, int *row2slot);

@@ -176,6 +176,7 @@ __device__ __forceinline__ void reset_ffn_control(int *early_flag, int n_words, 
   if (threadIdx.x == 0) {
     unit_counter[0] = 0;
     unit_counter[1] = 0;
+    unit_counter[2] = 0;
   }
   if (fence_reset) {
     __threadfence();
@@ -495,6 +496,8 @@ struct RouteArgs {
   int ffn_ctas;                 // CTAs of the FFN kernel: CTA c starts on gate/up unit c of the list
   int rows_later;               // the row of every (token, slot) pair is left to the row kernel (large trees)
   int res_first, res_count;     // experts resident on this GPU (expert-parallel shard); res_count = N: all
+  int chunk;                    // most token rows per work unit
+  int rank_order;               // 1: the unit list follows the shortlist's rank order also for many tokens
   int dense_all;                // gate/up units are marked "all tokens from hidden" (trees of at most 16 tokens)
 };
 
@@ -736,7 +739,7 @@ __global__ void __launch_bounds__(kRouteWarps * 32) route_kernel(RouteArgs a) {
       for (int i = tid; i < N * used_words; i += blockDim.x) s_colmask[i] = __ldcg(ws.colmask + i);
     // work units and the active count cover the resident experts only; rows and offsets cover all
     const bool resident = tid >= a.res_first && tid < a.res_first + a.res_count;
-    const int chunks = resident ? (c + kMaxTokChunk - 1) / kMaxTokChunk : 0;
+    const int chunks = resident ? (c + a.chunk - 1) / a.chunk : 0;
     // rows in bits 0..23, chunks in bits 24..43, active flag in bits 44..
     const unsigned long long v = (unsigned long long)c | ((unsigned long long)chunks << 24) |
                                  ((unsigned long long)(c > 0 && resident) << 44);
@@ -801,7 +804,7 @@ __global__ void __launch_bounds__(kRouteWarps * 32) route_kernel(RouteArgs a) {
       s_nchunks = tot;
     }
     __syncthreads();
-  } else if (a.tiles_up > 0 && M <= 2 * kMaxTokChunk) {
+  } else if (a.tiles_up > 0 && (M <= 2 * kMaxTokChunk || a.rank_order)) {
     // Trees of up to 256 tokens without early start: the listed experts in the shortlist's rank order too, each
     // with its one or two token chunks.  Rank order is roughly row-count order, so the units that take longest
     // (two full chunks, whose slabs are read twice) are handed out first and the list ends with cheap ones; in
@@ -906,8 +909,8 @@ __global__ void __launch_bounds__(kRouteWarps * 32) route_kernel(RouteArgs a) {
         const int chunks_e = s_cand[e];
         const int local = v - s_unit_base[e] * tiles;
         const int tl = local / chunks_e, c = local - tl * chunks_e;
-        const int row0 = s_offset[e] + c * kMaxTokChunk;
-        const int rows = min(kMaxTokChunk, s_count[e] - c * kMaxTokChunk);
+        const int row0 = s_offset[e] + c * a.chunk;
+        const int rows = min(a.chunk, s_count[e] - c * a.chunk);
         ws.units[u] = Unit{e, tl, row0, rows, s_unit_base[e] + c, phase, (a.dense_all && !phase) ? 2 : 0, 0};
       }
     }
@@ -963,6 +966,8 @@ static cudaError_t launch_route_kernel(const LaunchCtx &c, const float *logits) 
   a.early = c.ru > 0 ? c.early : 0;
   a.ffn_ctas = tc_grid_size(D.device);
   a.rows_later = rows_in_row_kernel(c.M);
+  a.chunk = c.chunk;
+  a.rank_order = c.rank_order;
   a.dense_all = c.ru > 0 ? c.dense_all : 0;
   a.res_first = c.res_count > 0 ? c.res_first : 0;
   a.res_count = c.res_count > 0 ? c.res_count : D.n_experts;

@@ -291,6 +291,7 @@ class Layer:
 
     KERNEL_NAMES_TC = ("router_topk", "route", "gather", "ffn")
     KERNEL_NAMES_TC_SMALL = ("router_topk", "route", "ffn")      # trees of at most 16 tokens, CUDA-core layers
+    KERNEL_NAMES_PAIR = ("router_topk", "route", "gather", "ffn_gate_up", "ffn_down", "combine")     # many tokens
 
     def debug_set_wait(self, limit_cycles: int, ready_bias: int):
         """Test hook: bound of the device-side waits and a ready-counter bias that makes them run out."""
@@ -305,7 +306,7 @@ class Layer:
         n = C.c_int(0)
         _check(lib().moespec_get_kernel_times(self._h, C.cast(ms, C.c_void_p), 8, C.cast(C.byref(n), C.c_void_p)),
                "moespec_get_kernel_times")
-        names = self.KERNEL_NAMES_TC_SMALL if n.value == 3 else self.KERNEL_NAMES_TC
+        names = {3: self.KERNEL_NAMES_TC_SMALL, 6: self.KERNEL_NAMES_PAIR}.get(n.value, self.KERNEL_NAMES_TC)
         return {names[i]: float(ms[i]) for i in range(min(n.value, len(names)))}
 
     def last_launch_count(self) -> int:

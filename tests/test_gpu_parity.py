@@ -142,6 +142,26 @@ def test_cuda_core_ffn_row_counts(dtype):
         assert st["n_rows"] == 3 * M          # every expert has all M rows
 
 
+# ------------------------------------------------------------------ SM-pair FFN at the edges of its tiles
+@pytest.mark.parametrize("dtype", ["bf16", "fp16"])
+def test_pair_ffn_row_counts(dtype):
+    """Trees beyond 256 tokens with many rows per expert: last chunks of 1, 64, 65, 128, 129, 191 and 256 rows (one and
+    two accumulator slots, every box height), one to four chunks, widths of one and three tiles, residual and 16-bit
+    outputs.  Tolerance: the suite's bars for 16-bit intermediates."""
+    for d, f in [(256, 768), (768, 256)]:
+        cfg = synth.CONFIGS["olmoe"].with_(d=d, f=f, n_experts=3, k=3, dtype=dtype)
+        for M in [257, 320, 321, 384, 385, 447, 512, 513, 900]:
+            case = H.make_case(cfg, M, M)
+            layer = make_layer(case, max_M=M, max_k=3, out_dtype=torch.float32)
+            _, _, st = run_e2e(cfg, M, 3, orc.SUBSTITUTION, orc.FROM_ALL, True, ms().FFN_AUTO, case=case, layer=layer)
+            assert st["n_rows"] == 3 * M and layer.last_launch_count() >= 6
+            layer.destroy()
+    cfg = synth.CONFIGS["olmoe"].with_(d=512, f=512, n_experts=24, k=4, dtype=dtype)
+    out16 = synth.torch_dtype(dtype)
+    run_e2e(cfg, 700, 9, orc.TRUNCATION, orc.FROM_UNION, False, ms().FFN_AUTO, seed=1)
+    run_e2e(cfg, 600, 12, orc.SUBSTITUTION, orc.FROM_ALL, True, ms().FFN_AUTO, seed=2, residual=True, out_dtype=out16)
+
+
 # ------------------------------------------------------------------ integer half, bit exact
 ROUTE_SHAPES = [
     ("tiny", dict(), [1, 15], [1, 2, 4, 8, 16, 40]),
