@@ -34,6 +34,7 @@ struct moespec_layer {
   TcMaps maps;
   int last_M, last_k;
   int last_launches;
+  int last_timed;       // steps of the last verify call that profiling brackets with events (router kernels as one)
   bool profiling;
   cudaEvent_t ev[kMaxProfiled + 1];
   // host-buffer entry point: the copy-in, the kernels and the copy-out as one instantiated graph
@@ -311,7 +312,8 @@ int run_layer(moespec_layer *L, const void *hidden, int M, int k, int B, void *o
   }
   L->last_M = M;
   L->last_k = k;
-  L->last_launches = launches;
+  L->last_launches = launches + router_launches(c) - 1;
+  L->last_timed = launches;
   return MOESPEC_OK;
 }
 
@@ -562,7 +564,8 @@ int moespec_calibrate(moespec_layer_t *L, const void *hidden, int M, int k, void
   if (e != cudaSuccess) return cuda_fail(e);
   L->last_M = M;
   L->last_k = k;
-  L->last_launches = 2;
+  L->last_launches = router_launches(c) + 1;
+  L->last_timed = 0;
   return MOESPEC_OK;
 }
 
@@ -650,6 +653,7 @@ int moespec_route_from_logits(moespec_layer_t *L, const float *logits, int M, in
   if (e != cudaSuccess) return cuda_fail(e);
   L->last_M = M;
   L->last_k = k;
+  L->last_timed = 0;
   L->last_launches = M > kMaxTokChunk ? 3 : 2;      // large trees add the row kernel
   return MOESPEC_OK;
 }
@@ -746,10 +750,10 @@ int moespec_set_profiling(moespec_layer_t *L, int on) {
 int moespec_get_kernel_times(moespec_layer_t *L, float *ms, int capacity, int *n_kernels) {
   if (!is_live(L)) return MOESPEC_ERR_BAD_HANDLE;
   if (!ms || !n_kernels) return MOESPEC_ERR_NULL_POINTER;
-  if (!L->profiling || L->last_launches <= 1) return MOESPEC_ERR_INVALID_ARG;
+  if (!L->profiling || L->last_timed < 1) return MOESPEC_ERR_INVALID_ARG;
   DeviceGuard guard(L->desc.device);
   if (guard.err != cudaSuccess) return cuda_fail(guard.err);
-  const int n = L->last_launches < kMaxProfiled ? L->last_launches : kMaxProfiled;
+  const int n = L->last_timed < kMaxProfiled ? L->last_timed : kMaxProfiled;
   cudaError_t e = cudaEventSynchronize(L->ev[n]);
   if (e != cudaSuccess) return cuda_fail(e);
   *n_kernels = n;

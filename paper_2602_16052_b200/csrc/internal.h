@@ -140,6 +140,7 @@ cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_
 
 // routing.cu
 cudaError_t launch_router_logits(const LaunchCtx &c, const void *hidden);
+int router_launches(const LaunchCtx &c);                             // kernels launch_router_logits enqueues
 cudaError_t launch_route(const LaunchCtx &c, const float *logits);   // softmax/top-k kernel + route kernel
 cudaError_t launch_route_after_router(const LaunchCtx &c);           // route kernel only
 cudaError_t launch_calib_accumulate(const LaunchCtx &c);             // c_i += natural counts of the last router launch

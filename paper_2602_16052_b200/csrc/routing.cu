@@ -394,6 +394,79 @@ __global__ void __launch_bounds__(NW * 32) router_mma_kernel(const T *__restrict
   }
 }
 
+// ---------------------------------------------------------------------------
+// K1 for many tokens, logits only: the same dot products (same K ranges per warp, same MMA order, partial tiles added
+// in warp order: the same logits) with 64 experts x 16 tokens per CTA, so that the router matrix is fetched once per
+// 16 tokens instead of once per 8 and the CTAs are one wave at 2048 tokens.  Softmax and top-k follow in
+// softmax_topk_kernel, one warp per token.  What bounded the kernel above there was its waves: 1024 CTAs, one per SM,
+// each a chain of loads, exchange, arrival counter and softmax (us between events, 64 experts, before / now: 1024
+// tokens 29 / 22, 1500 36 / 25, 2048 44 / 27; 128 experts, 1000 tokens 42 / 30).
+// ---------------------------------------------------------------------------
+constexpr int kRgExperts = 64, kRgTokens = 16, kRgWarps = 16;
+
+template <typename T>
+__global__ void __launch_bounds__(kRgWarps * 32) router_gemm_kernel(const T *__restrict__ hidden, const T *__restrict__ Wr,
+                                                                    const float *__restrict__ bias, float *logits,
+                                                                    int *early_flag, int *unit_counter, int M, int N,
+                                                                    int d) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int g = lane >> 2, tg = lane & 3;
+  const int e0 = blockIdx.x * kRgExperts, t0 = blockIdx.y * kRgTokens;
+  __shared__ float s_part[kRgWarps][kRgExperts * 8];
+  const int kw = d / kRgWarps;                            // K range of this warp: [warp*kw, warp*kw + kw)
+  const int col = warp * kw + tg * 8;
+  int wr[8], hr[2];                                       // rows beyond N or M repeat the last one and are not stored
+#pragma unroll
+  for (int r = 0; r < 8; ++r) wr[r] = min(e0 + r * 8 + g, N - 1) * d + col;
+#pragma unroll
+  for (int r = 0; r < 2; ++r) hr[r] = min(t0 + r * 8 + g, M - 1) * d + col;
+  float c[4][2][4] = {};
+  uint4 A[8], B[2];
+#pragma unroll
+  for (int r = 0; r < 8; ++r) A[r] = *reinterpret_cast<const uint4 *>(Wr + wr[r]);      // a constant of the layer
+  pdl_wait();          // hidden may be the previous layer's output; the workspace is still in use until then
+  reset_ffn_control(early_flag, N, unit_counter, 0);
+  pdl_trigger();
+#pragma unroll
+  for (int r = 0; r < 2; ++r) B[r] = *reinterpret_cast<const uint4 *>(hidden + hr[r]);
+  for (int k0 = 0; k0 < kw; k0 += 32) {
+    uint4 An[8], Bn[2];
+    if (k0 + 32 < kw) {
+#pragma unroll
+      for (int r = 0; r < 8; ++r) An[r] = *reinterpret_cast<const uint4 *>(Wr + wr[r] + k0 + 32);
+#pragma unroll
+      for (int r = 0; r < 2; ++r) Bn[r] = *reinterpret_cast<const uint4 *>(hidden + hr[r] + k0 + 32);
+    }
+#pragma unroll
+    for (int m = 0; m < 4; ++m)
+#pragma unroll
+      for (int n = 0; n < 2; ++n) {
+        mma_16816(c[m][n], A[2 * m].x, A[2 * m + 1].x, A[2 * m].y, A[2 * m + 1].y, B[n].x, B[n].y, T());
+        mma_16816(c[m][n], A[2 * m].z, A[2 * m + 1].z, A[2 * m].w, A[2 * m + 1].w, B[n].z, B[n].w, T());
+      }
+#pragma unroll
+    for (int r = 0; r < 8; ++r) A[r] = An[r];
+#pragma unroll
+    for (int r = 0; r < 2; ++r) B[r] = Bn[r];
+  }
+#pragma unroll
+  for (int n = 0; n < 2; ++n) {                           // eight tokens at a time through shared memory
+    if (n > 0) __syncthreads();
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      float *p = s_part[warp] + (m * 16 + g) * 8 + 2 * tg;
+      *reinterpret_cast<float2 *>(p) = make_float2(c[m][n][0], c[m][n][1]);
+      *reinterpret_cast<float2 *>(p + 64) = make_float2(c[m][n][2], c[m][n][3]);
+    }
+    __syncthreads();
+    const int tl = threadIdx.x & 7, el = threadIdx.x >> 3, t = t0 + n * 8 + tl;
+    float acc = 0.f;
+#pragma unroll
+    for (int w = 0; w < kRgWarps; ++w) acc += s_part[w][threadIdx.x];
+    if (e0 + el < N && t < M) logits[(size_t)t * N + e0 + el] = acc + (bias ? bias[e0 + el] : 0.f);
+  }
+}
+
 template <typename T, int NW = 8>
 static cudaError_t launch_router_mma(const LaunchCtx &c, const void *hidden) {
   const moespec_layer_desc &D = *c.desc;
@@ -418,8 +491,28 @@ static bool use_router_mma(const LaunchCtx &c) {
   return !off && is_16bit(c.desc->dtype) && (c.M >= min_m || c.desc->n_experts >= 128) && c.desc->d % 256 == 0;
 }
 
+static cudaError_t launch_softmax_topk(const LaunchCtx &c, const float *logits, int *early_flag);
+
+// Many tokens: logits by the 64 x 16 kernel, softmax and top-k by one warp per token.  us between events, one kernel /
+// two: 512 tokens 19.6 / 22.1 (too few CTAs), 1024 28.8 / 21.6; the line lies between.
+static bool use_router_gemm(const LaunchCtx &c) { return use_router_mma(c) && c.M >= 768 && c.desc->d % 512 == 0; }
+
+template <typename T>
+static cudaError_t launch_router_gemm(const LaunchCtx &c, const void *hidden) {
+  const moespec_layer_desc &D = *c.desc;
+  const Workspace &ws = *c.ws;
+  const dim3 grid((D.n_experts + kRgExperts - 1) / kRgExperts, (c.M + kRgTokens - 1) / kRgTokens);
+  cudaError_t e = launch_kernel(router_gemm_kernel<T>, grid, dim3(kRgWarps * 32), 0, c.stream, (const T *)hidden,
+                                (const T *)D.router_w, D.router_bias, ws.logits, ws.early_flag, ws.unit_counter, c.M,
+                                D.n_experts, D.d);
+  return e == cudaSuccess ? launch_softmax_topk(c, ws.logits, nullptr) : e;
+}
+template <>
+cudaError_t launch_router_gemm<float>(const LaunchCtx &, const void *) { return cudaErrorNotSupported; }
+
 template <typename T>
 static cudaError_t launch_router_t(const LaunchCtx &c, const void *hidden) {
+  if (use_router_gemm(c)) return launch_router_gemm<T>(c, hidden);
   // sixteen warps per CTA where K splits sixteen ways into whole 32-element steps: the eight tokens of a tile
   // then get their softmax and their top-k on separate warps (2.5 µs per layer less than eight warps at
   // 65 to 255 tokens and for 128 experts)
@@ -451,6 +544,8 @@ static cudaError_t launch_router_t(const LaunchCtx &c, const void *hidden) {
                          ws.colmask, c.M, D.n_experts, D.d, c.k);
 }
 
+int router_launches(const LaunchCtx &c) { return use_router_gemm(c) ? 2 : 1; }
+
 cudaError_t launch_router_logits(const LaunchCtx &c, const void *hidden) {
   if (c.desc->dtype == MOESPEC_BF16) return launch_router_t<__nv_bfloat16>(c, hidden);
   if (c.desc->dtype == MOESPEC_FP16) return launch_router_t<__half>(c, hidden);
@@ -470,6 +565,12 @@ __global__ void __launch_bounds__(128) softmax_topk_kernel(const float *logits, 
   if (t < M)
     token_phase(logits + (size_t)t * N, N, k, prob + (size_t)t * N, topk_idx + (size_t)t * k, score_fx, natcnt,
                 threadIdx.x & 31);
+}
+
+static cudaError_t launch_softmax_topk(const LaunchCtx &c, const float *logits, int *early_flag) {
+  return launch_kernel(softmax_topk_kernel, dim3((c.M + 3) / 4), dim3(128), 0, c.stream, logits, c.ws->prob,
+                       c.ws->topk_idx, c.ws->score_fx, c.ws->natcnt_acc, early_flag, c.ws->colmask, c.M,
+                       c.desc->n_experts, c.k);
 }
 
 __device__ __forceinline__ double shfl_double(double x, int src) {
@@ -1001,9 +1102,7 @@ cudaError_t launch_route_after_router(const LaunchCtx &c) { return launch_route_
 
 // Routing from caller-supplied logits: per-token softmax/top-k first (two launches).
 cudaError_t launch_route(const LaunchCtx &c, const float *logits) {
-  cudaError_t e = launch_kernel(softmax_topk_kernel, dim3((c.M + 3) / 4), dim3(128), 0, c.stream, logits, c.ws->prob,
-                                c.ws->topk_idx, c.ws->score_fx, c.ws->natcnt_acc, c.ws->early_flag, c.ws->colmask, c.M,
-                                c.desc->n_experts, c.k);
+  cudaError_t e = launch_softmax_topk(c, logits, c.ws->early_flag);
   if (e != cudaSuccess) return e;
   e = launch_route_kernel(c, logits);
   if (e != cudaSuccess || !rows_in_row_kernel(c.M)) return e;
@@ -1125,6 +1224,8 @@ cudaError_t routing_configure() {
   set((const void *)router_topk_kernel<float, 2>);
   set((const void *)router_topk_kernel<float, 4>);
   set((const void *)router_topk_kernel<float, 8>);
+  set((const void *)router_gemm_kernel<__nv_bfloat16>);
+  set((const void *)router_gemm_kernel<__half>);
   set((const void *)softmax_topk_kernel);
   set((const void *)route_kernel<1>);
   set((const void *)route_kernel<2>);

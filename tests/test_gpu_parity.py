@@ -162,6 +162,53 @@ def test_pair_ffn_row_counts(dtype):
     run_e2e(cfg, 600, 12, orc.SUBSTITUTION, orc.FROM_ALL, True, ms().FFN_AUTO, seed=2, residual=True, out_dtype=out16)
 
 
+def test_pair_ffn_in_captured_graphs():
+    """The SM-pair launches replayed from the stack's and the host entry point's graphs, bit for bit as enqueued; with
+    an expired wait the status says so and the next call is unharmed."""
+    m = ms()
+    cfg = synth.CONFIGS["olmoe"].with_(d=256, f=256, n_experts=8, k=4)
+    M, B = 300, 6
+    cases = [H.make_case(cfg, M, 1, layer=l) for l in range(2)]
+    layers = [make_layer(c, max_M=M, max_k=4, residual=True) for c in cases]
+    stack = m.Stack(layers)
+    h = cases[0]["hidden"]
+    out = stack.verify_stack(h, 4, B).clone()
+    assert stack.last_launch_count() == 12
+    stack.set_graph(False)
+    assert torch.equal(out, stack.verify_stack(h, 4, B))
+    step = layers[0].verify_layer(h, 4, B)
+    assert torch.equal(out, layers[1].verify_layer(step, 4, B))
+    hh, oh = h.cpu().pin_memory(), torch.empty_like(h, device="cpu").pin_memory()
+    assert torch.equal(layers[0].verify_layer_host(hh, 4, B, oh), step.cpu())
+    layers[0].debug_set_wait(2_000_000, 1)
+    layers[0].verify_layer(h, 4, B)
+    assert layers[0].get_stats()["status"] == m.ERR_TIMEOUT
+    layers[0].debug_set_wait(0, 0)
+    assert torch.equal(layers[0].verify_layer(h, 4, B), step) and layers[0].get_stats()["status"] == 0
+    stack.destroy()
+
+
+# ------------------------------------------------------------------ router of many tokens
+@pytest.mark.parametrize("dtype", ["bf16", "fp16"])
+def test_router_of_many_tokens(dtype):
+    """The 64 x 16 router tile at its edges: the smallest tree it takes, token counts that are not multiples of 8 or
+    16, expert counts below, at and above one tile, one and several K steps per warp.  Logits against fp64 within the
+    suite's bound (2e-5 of the largest), routing on them bit for bit.  (Not the output: with 4 experts of f = 128 the
+    largest of 400 000 errors of the bf16 intermediate is 0.023 RMS whatever the router does: half an ulp of 2^-9 in
+    each of 4 x 128 products, times the 5 sigma that a maximum over so many reaches.)"""
+    for M, N, d in [(768, 64, 512), (769, 33, 1024), (777, 65, 512), (1000, 128, 512), (791, 3, 2048)]:
+        cfg = synth.CONFIGS["olmoe"].with_(d=d, f=128, n_experts=N, k=min(4, N), dtype=dtype)
+        case = H.make_case(cfg, M, N)
+        layer = make_layer(case, max_M=M, max_k=cfg.k)
+        layer.verify_layer(case["hidden"], cfg.k, max(1, N // 2))
+        z = layer.get_logits()
+        z_ref = orc.router_logits(H.f64(case["hidden"]), H.f64(case["router_w"]), H.f64(case["router_bias"]))
+        assert np.max(np.abs(z - z_ref)) <= 2e-5 * max(1.0, np.abs(z_ref).max())
+        r = H.oracle_route(z, cfg.k, max(1, N // 2), orc.SUBSTITUTION, orc.FROM_ALL, True)
+        H.compare_routing(layer.get_routing(), r, orc.SUBSTITUTION, cfg.k)
+        layer.destroy()
+
+
 # ------------------------------------------------------------------ integer half, bit exact
 ROUTE_SHAPES = [
     ("tiny", dict(), [1, 15], [1, 2, 4, 8, 16, 40]),
