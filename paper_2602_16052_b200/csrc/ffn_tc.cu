@@ -26,11 +26,11 @@
 // circular wait, however the grid is placed on the SMs (a CTA that becomes
 // resident late simply draws a later ticket, e.g. when another handle's kernel
 // holds some of the SMs).  The dispenser and the down-unit counter are zeroed
-// by the router kernel of the call, which completes before this kernel starts.
+// by the router kernel of the call before this kernel can start.
 //
 // Early start (trees of up to 128 tokens): the CTAs of this kernel are resident
 // while the routing kernels still run.  A CTA whose first ticket c is below the
-// grid size does not wait for them: as soon as the routing kernel has published
+// grid size does not wait for them: as soon as they have published
 // the shortlist (a flag; at once when the shortlist is fixed) it starts on
 // gate/up unit c of the rank-ordered list -- expert S_rank[c / slabs], slab
 // c % slabs -- with ALL tokens of the tree as the B operand, read from `hidden`
@@ -277,7 +277,8 @@ __device__ __forceinline__ bool epilogue_any(bool failed) {
   return any != 0;
 }
 
-__global__ void __launch_bounds__(kThreads, 1) ffn_tc_kernel(const __grid_constant__ TcMapsCall maps, TcArgs a) {
+// At most 80 registers: the next call's tree_router_kernel (8 warps of 136) then fits beside this kernel's CTAs.
+__global__ void __maxnreg__(80) ffn_tc_kernel(const __grid_constant__ TcMapsCall maps, TcArgs a) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   // stages first (1024-byte aligned for the 128-byte swizzle), control block after
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -300,8 +301,8 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_tc_kernel(const __grid_consta
   const int n_stages = a.n_stages;
   pdl_trigger();
   // The first ticket and, with early start, the first 32 shortlist words are requested before anything else:
-  // their round trips through L2 overlap the set-up below.  (The router kernel of this call left the
-  // dispenser at zero and has completed, or with a fixed shortlist has at least performed that reset.)
+  // their round trips through L2 overlap the set-up below.  (The router kernel of this call has zeroed the
+  // dispenser: it has completed, or has at least performed that reset before this kernel was released.)
   int t_first = 0, w_pre = 0;
   if (warp == 0) {
     if (lane == 0) t_first = atomicAdd(a.unit_counter, 1);
@@ -367,7 +368,7 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_tc_kernel(const __grid_consta
       return x;
     };
     if (a.early) {
-      // The routing kernel publishes the shortlist long before the gather order exists.  Ticket c below the
+      // The shortlist is published long before the gather order exists.  Ticket c below the
       // grid size is gate/up unit c of the rank-ordered list (expert S_rank[c / tiles], slab c % tiles) and
       // is started on with ALL tokens as the MMA's N dimension, read straight from `hidden`; the epilogue
       // keeps the routed tokens only.  The routing kernel builds the unit list in the same order and keeps

@@ -5,13 +5,14 @@
 // per-expert gather order (Appendix C).
 //
 // Three launches:
-//   router_topk_kernel   router dot products; the CTA that finishes a token
+//   tree_router_kernel   router dot products, softmax, top-k and scores of small trees, and the shortlist for the FFN kernel
+//   router_topk_kernel   the same without the shortlist, for the layers that one does not take; the CTA that finishes a token
 //                        tile's last logit also runs those tokens' softmax and
 //                        top-k and adds their probabilities to the per-expert
 //                        scores (a counter, never a wait).  router_mma_kernel is
 //                        the same on the tensor cores, for larger trees.
 //   route_kernel         eight tokens per CTA: every CTA ranks the scores itself
-//                        (shortlist; CTA 0 publishes it for the FFN kernel),
+//                        (shortlist; CTA 0 publishes it for the FFN kernel unless the router has),
 //                        re-routes its tokens, and the CTA that finishes last
 //                        does the scan, the gather order, the work-unit list and
 //                        the statistics
@@ -24,6 +25,7 @@
 #include "internal.h"
 #include <cstdlib>
 #include <math_constants.h>
+#include <type_traits>
 
 namespace moespec {
 
@@ -76,40 +78,56 @@ __device__ __forceinline__ int warp_take_best(const uint32_t (&key)[W], uint32_t
   return mine;
 }
 
+// Softmax of one token by one warp (Eq. 1, fp64); lane l owns experts l, l+32, ..., whose logits are in v (-inf beyond
+// the N-th).  The exponentials of a lane are independent chains, not branches, so that they overlap.
+template <int W>
+__device__ __forceinline__ void softmax_row(const float (&v)[W], int N, double (&p)[W]) {
+  float mx = -CUDART_INF_F;
+#pragma unroll
+  for (int s = 0; s < W; ++s) mx = fmaxf(mx, v[s]);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(kFull, mx, o));
+  double sum = 0.0;
+#pragma unroll
+  for (int s = 0; s < W; ++s) p[s] = exp((double)v[s] - (double)mx);
+#pragma unroll
+  for (int s = 0; s < W; ++s) sum += p[s];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(kFull, sum, o);
+  // p / sum by one division: the quotient from the rounded reciprocal is off by an ulp at most, and the exact remainder
+  // corrects it to the rounded quotient (Markstein 1990).  A division for each p took its slow path for every p that is
+  // zero: 965 cycles for a row of 16 experts, 542 this way.
+  const double r = 1.0 / sum;
+#pragma unroll
+  for (int s = 0; s < W; ++s) {
+    const double q = p[s] * r;
+    p[s] = fma(fma(-q, sum, p[s]), r, q);
+  }
+}
+
+// A probability's addend to its expert's score.  p == 1 exactly is clamped one unit below 2^52, so that max_M = 4096 such
+// tokens cannot wrap the sum.
+__device__ __forceinline__ unsigned long long fixed_point(double p) {
+  return min((unsigned long long)__double2ull_rn(p * kScoreScale), kScoreOneMinus);
+}
+
 // Softmax of one token by one warp (Eq. 1, fp64); adds the probabilities to the per-expert scores (Eq. 5).
+// A token's logits: written by other CTAs of the launch, they are read through L2; in shared memory they are this CTA's.
+__device__ __forceinline__ float load_logit(const float *z) { return __isShared(z) ? *z : __ldcg(z); }
+
 template <int W>
 __device__ __forceinline__ void token_softmax(const float *zrow, int N, double *prob_row, unsigned long long *score_fx,
                                               int lane) {
   float v[W];
-  uint32_t valid = 0;
-  float mx = -CUDART_INF_F;
 #pragma unroll
-  for (int s = 0; s < W; ++s) {
-    const int idx = lane + 32 * s;
-    v[s] = -CUDART_INF_F;
-    if (idx < N) {
-      v[s] = __ldcg(zrow + idx);          // written by other CTAs of this launch: read through L2
-      valid |= 1u << s;
-      mx = fmaxf(mx, v[s]);
-    }
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(kFull, mx, o));
-  double e[W], sum = 0.0;
-#pragma unroll
-  for (int s = 0; s < W; ++s) {
-    e[s] = 0.0;
-    if ((valid >> s) & 1u) { e[s] = exp((double)v[s] - (double)mx); sum += e[s]; }
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(kFull, sum, o);
+  for (int s = 0; s < W; ++s) v[s] = lane + 32 * s < N ? load_logit(zrow + lane + 32 * s) : -CUDART_INF_F;
+  double p[W];
+  softmax_row<W>(v, N, p);
 #pragma unroll
   for (int s = 0; s < W; ++s)
-    if ((valid >> s) & 1u) {
-      const double p = e[s] / sum;
-      prob_row[lane + 32 * s] = p;
-      // p == 1 exactly is clamped one unit below 2^52, so that max_M = 4096 such tokens cannot wrap the sum
-      atomicAdd(score_fx + lane + 32 * s, min((unsigned long long)__double2ull_rn(p * kScoreScale), kScoreOneMinus));
+    if (lane + 32 * s < N) {
+      prob_row[lane + 32 * s] = p[s];
+      atomicAdd(score_fx + lane + 32 * s, fixed_point(p[s]));
     }
 }
 
@@ -123,7 +141,7 @@ __device__ __forceinline__ void token_topk(const float *zrow, int N, int k, int 
     const int idx = lane + 32 * s;
     key[s] = 0;
     if (idx < N) {
-      key[s] = order_key(__ldcg(zrow + idx));
+      key[s] = order_key(load_logit(zrow + idx));
       valid |= 1u << s;
     }
   }
@@ -165,13 +183,13 @@ __device__ __forceinline__ void clear_colmask(unsigned *colmask, int words) {
 }
 
 // The FFN kernel's control words must be in their initial state when its first CTA starts: the shortlist words
-// at 0 (the routing kernel publishes the call's shortlist later; the FFN kernel's CTAs poll them), its unit
-// dispenser and its down-unit counter at 0.  The router kernel's first CTA sets them: it runs after the
-// previous call's FFN kernel has completed (it has just waited for that) and completes before this call's FFN
-// kernel can start -- except with a fixed shortlist, where the FFN kernel is released right behind this kernel's
-// CTAs: there the stores are performed (fence) before this CTA releases the dependents.
+// at 0 (the call's shortlist is published later; the FFN kernel's CTAs poll them), its unit dispenser and its
+// down-unit counter at 0.  One CTA of the router kernel sets them: it runs after the previous call's FFN kernel has
+// completed (it has just waited for that) and completes before this call's FFN kernel can start -- except where the
+// FFN kernel is released right behind the router kernel's CTAs (a fixed shortlist, or tree_router_kernel): there the
+// stores are performed (fence) before this CTA releases the dependents.
 __device__ __forceinline__ void reset_ffn_control(int *early_flag, int n_words, int *unit_counter, int fence_reset) {
-  if (!early_flag || blockIdx.x != 0 || blockIdx.y != 0) return;
+  if (!early_flag) return;
   for (int i = threadIdx.x; i < n_words; i += blockDim.x) early_flag[i] = 0;
   if (threadIdx.x == 0) {
     unit_counter[0] = 0;
@@ -182,6 +200,29 @@ __device__ __forceinline__ void reset_ffn_control(int *early_flag, int n_words, 
     __threadfence();
     __syncthreads();
   }
+}
+
+// A load that stays where it is written: before a dependency wait, that is.  (The compiler moves plain loads of constant
+// data behind it, next to their first use.)
+__device__ __forceinline__ uint4 load_early(const void *p) {
+  uint4 v;
+  asm volatile("ld.global.nc.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ float load_early(const float *p) {
+  float v;
+  asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// The same variable in CTA `rank` of the cluster.
+__device__ __forceinline__ void st_cluster(void *p, uint32_t rank, uint32_t v) {
+  uint32_t addr;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(addr) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+  asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
 
 // ---------------------------------------------------------------------------
@@ -215,7 +256,7 @@ __global__ void __launch_bounds__(256) router_topk_kernel(const T *__restrict__ 
       if ((lane + u * 32) * VEC < d) rw[u] = *reinterpret_cast<const uint4 *>(Wr + (size_t)i * d + (lane + u * 32) * VEC);
   }
   pdl_wait();          // hidden may be the previous layer's output; the workspace is still in use until then
-  reset_ffn_control(early_flag, N, unit_counter, fence_reset);
+  if (blockIdx.x == 0 && blockIdx.y == 0) reset_ffn_control(early_flag, N, unit_counter, fence_reset);
   // Dependents are released only now: with a fixed shortlist the FFN kernel of this call starts at once,
   // and it reads `hidden`, which the previous kernel in the stream may have produced.
   pdl_trigger();
@@ -339,7 +380,7 @@ __global__ void __launch_bounds__(NW * 32) router_mma_kernel(const T *__restrict
     }
   }
   pdl_wait();          // hidden may be the previous layer's output; the workspace is still in use until then
-  reset_ffn_control(early_flag, N, unit_counter, fence_reset);
+  if (blockIdx.x == 0 && blockIdx.y == 0) reset_ffn_control(early_flag, N, unit_counter, fence_reset);
   pdl_trigger();       // released only now: see router_topk_kernel
   clear_colmask(colmask, N * ((M + 31) >> 5));
   const T *hb = hidden + (size_t)min(t0 + g, M - 1) * d + warp * kw + tg * 8;
@@ -425,7 +466,7 @@ __global__ void __launch_bounds__(kRgWarps * 32) router_gemm_kernel(const T *__r
 #pragma unroll
   for (int r = 0; r < 8; ++r) A[r] = *reinterpret_cast<const uint4 *>(Wr + wr[r]);      // a constant of the layer
   pdl_wait();          // hidden may be the previous layer's output; the workspace is still in use until then
-  reset_ffn_control(early_flag, N, unit_counter, 0);
+  if (blockIdx.x == 0 && blockIdx.y == 0) reset_ffn_control(early_flag, N, unit_counter, 0);
   pdl_trigger();
 #pragma unroll
   for (int r = 0; r < 2; ++r) B[r] = *reinterpret_cast<const uint4 *>(hidden + hr[r]);
@@ -492,6 +533,8 @@ static bool use_router_mma(const LaunchCtx &c) {
 }
 
 static cudaError_t launch_softmax_topk(const LaunchCtx &c, const float *logits, int *early_flag);
+static bool tree_router_takes(const LaunchCtx &c);
+static cudaError_t launch_router_for_tree(const LaunchCtx &c, const void *hidden);
 
 // Many tokens: logits by the 64 x 16 kernel, softmax and top-k by one warp per token.  us between events, one kernel /
 // two, 64 experts of d = 2048: 512 tokens 19.6 / 22.1 (too few CTAs), 768 23.6 / 21.6, 1024 28.8 / 21.6.  Up to 32 experts
@@ -548,9 +591,10 @@ static cudaError_t launch_router_t(const LaunchCtx &c, const void *hidden) {
                          ws.colmask, c.M, D.n_experts, D.d, c.k);
 }
 
-int router_launches(const LaunchCtx &c) { return use_router_gemm(c) ? 2 : 1; }
+int router_launches(const LaunchCtx &c) { return !tree_router_takes(c) && use_router_gemm(c) ? 2 : 1; }
 
 cudaError_t launch_router_logits(const LaunchCtx &c, const void *hidden) {
+  if (tree_router_takes(c)) return launch_router_for_tree(c, hidden);
   if (c.desc->dtype == MOESPEC_BF16) return launch_router_t<__nv_bfloat16>(c, hidden);
   if (c.desc->dtype == MOESPEC_FP16) return launch_router_t<__half>(c, hidden);
   return launch_router_t<float>(c, hidden);
@@ -603,10 +647,12 @@ struct RouteArgs {
   int res_first, res_count;     // experts resident on this GPU (expert-parallel shard); res_count = N: all
   int chunk;                    // most token rows per work unit
   int rank_order;               // 1: the unit list follows the shortlist's rank order also for many tokens
+  int from_router;              // the router kernel has published the shortlist and reset the FFN kernel's control words
   int dense_all;                // gate/up units are marked "all tokens from hidden" (trees of at most 16 tokens)
 };
 
 constexpr int kRouteWarps = 8;      // tokens per CTA of route_kernel
+constexpr int kMaxRouteWarps = 16;         // ... of any kernel that uses RouteShared
 constexpr int kColmaskCache = 1024; // words of the expert x token bit matrix the last CTA keeps in shared memory
 
 // Probability of expert `idx` from the row a warp holds in registers (lane l owns experts l, l+32, ...).
@@ -624,9 +670,11 @@ __device__ __forceinline__ double row_value(const double (&p)[W], int idx) {
 
 // Re-routing of one token (Eq. 7 / Eq. 8) with its mixing weights (Section 3.3); lane r owns slot r.
 // key[] / p[] are the token's logit keys and probabilities, valid says which slots exist.
-template <int W>
+// The kept experts are recorded in the call's accumulators, or (kOneCta) in the CTA's own bit matrix, one word per expert.
+template <int W, bool kOneCta = false>
 __device__ __forceinline__ void token_reroute(const RouteArgs &a, int t, int nS, const uint32_t *s_Smask,
-                                              const uint32_t (&key)[W], const double (&p)[W], int nat, int lane) {
+                                              const uint32_t (&key)[W], const double (&p)[W], int nat, int lane,
+                                              unsigned *s_colmask = nullptr, short *s_assign = nullptr) {
   const Workspace &ws = a.ws;
   const int k = a.k;
   const bool nat_kept = nat >= 0 && ((s_Smask[nat >> 5] >> (nat & 31)) & 1u);
@@ -672,17 +720,355 @@ __device__ __forceinline__ void token_reroute(const RouteArgs &a, int t, int nS,
   if (lane < k) {
     ws.assign_idx[(size_t)t * k + lane] = mine;
     ws.gate_w[(size_t)t * k + lane] = mine >= 0 ? (float)(p_mine / denom) : 0.f;
-    if (mine >= 0) {
+    if constexpr (kOneCta) {
+      s_assign[t * k + lane] = (short)mine;
+      if (mine >= 0) atomicOr(s_colmask + mine, 1u << t);
+    } else if (mine >= 0) {
       atomicAdd(ws.count_acc + mine, 1);
       atomicOr(ws.colmask + (size_t)mine * ((a.M + 31) >> 5) + (t >> 5), 1u << (t & 31));
     }
   }
 }
 
-template <int W>
-__device__ __forceinline__ void route_token(const RouteArgs &a, int t, int nS, const uint32_t *s_Smask,
-                                            const uint32_t (&key)[W], const double (&p)[W], int nat, int lane) {
-  token_reroute<W>(a, t, nS, s_Smask, key, p, nat, lane);
+// Shared memory of the shortlist, for up to NMAX experts, ...
+template <int NMAX>
+struct ShortlistShared {
+  unsigned long long score[NMAX];     // ranking key (score + 1, or 0 for a non-candidate)
+  int cand[NMAX];
+  int Srank[NMAX];
+  uint32_t Smask[kMaskWords];
+  unsigned long long warp_tot[kMaxRouteWarps];
+};
+// ... and of route_kernel, which stays below 16 KB, so that a CTA of the FFN kernel fits beside it.
+struct RouteShared : ShortlistShared<kMaxExperts> {
+  unsigned long long fx[kMaxExperts];        // fixed-point score
+  unsigned colmask[kColmaskCache];
+  int count[kMaxExperts];
+  int offset[kMaxExperts + 1];
+  int unit_base[kMaxExperts + 1];
+  int chunk_expert[kMaxExperts * 2];     // token chunk -> expert (first 2N chunks; more fall back)
+  int nactive, last, nchunks;
+  unsigned char all_dense[kMaxExperts];   // expert whose gate/up units all take every token from hidden
+};
+
+struct Shortlist {
+  int nS, nS_l, n_union;     // kept experts, those of them resident on this GPU (sh.Srank), size of the union
+};
+
+// Shortlist (Section 3.2) from the scores (Eq. 5) and the union (Eq. 3), which the caller's thread i < N has put into
+// sh.cand[i] and sh.score[i]; every thread of the CTA takes part.  write_rank, publish: this CTA also writes out the
+// shortlist, and publishes it to the FFN kernel.
+template <int NMAX>
+__device__ __forceinline__ Shortlist pick_shortlist(const RouteArgs &a, ShortlistShared<NMAX> &sh, int in_union,
+                                                    bool write_rank, bool publish) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n_warps = blockDim.x >> 5;
+  const int N = a.N;
+  const Workspace &ws = a.ws;
+  if (tid < kMaskWords) sh.Smask[tid] = 0u;
+  const int n_union = __syncthreads_count(in_union);
+  const int n_cand = __syncthreads_count(tid < N && sh.cand[tid]);
+  const bool fixed = a.shortlist == MOESPEC_STATIC;
+  const int nS = fixed ? min(a.B, ws.n_static) : min(a.B, n_cand);
+  if (fixed) {
+    // static ranking (Eq. 4): the shortlist is the first nS experts of the fixed ordering
+    if (tid < N) {
+      const int pos = ws.static_pos[tid];
+      if (pos < nS) {
+        sh.Srank[pos] = tid;
+        atomicOr(&sh.Smask[tid >> 5], 1u << (tid & 31));
+        if (write_rank) ws.S_rank[pos] = tid;
+      }
+    }
+  } else {
+    // Rank by counting, branch-free.  sh.score holds score+1 for candidates and 0 for the others, so a non-candidate
+    // never outranks a candidate.  2^gs threads share an expert, each takes every 2^gs-th of the others.
+    int gs = 0;
+    while ((N << (gs + 1)) <= (int)blockDim.x && gs < 3) ++gs;
+    const int i = tid >> gs, sub = tid & ((1 << gs) - 1);
+    const unsigned long long si = i < N ? sh.score[i] : 0ull;
+    int rank = 0;
+    if (i < N) {
+#pragma unroll 4
+      for (int j = sub; j < N; j += 1 << gs) {
+        const unsigned long long sj = sh.score[j];
+        rank += (int)((sj > si) | ((sj == si) & (j < i)));
+      }
+    }
+    for (int o = 1; o < (1 << gs); o <<= 1) rank += __shfl_xor_sync(kFull, rank, o);
+    if (i < N && sub == 0 && si != 0ull && rank < nS) {
+      sh.Srank[rank] = i;
+      atomicOr(&sh.Smask[i >> 5], 1u << (i & 31));
+      if (write_rank) ws.S_rank[rank] = i;
+    }
+  }
+  __syncthreads();
+  // What the FFN kernel works on is the part of the shortlist that is resident on this GPU, in rank order
+  // (all of it unless this layer is an expert-parallel shard): sh.Srank / nS_l from here on.  The shortlist
+  // itself stays in sh.Smask (re-routing) and in ws.S_rank.
+  const bool shard = a.res_count < N;
+  int nS_l = nS;
+  if (shard) {
+    int e_r = 0;
+    bool res = false;
+    if (tid < nS) {
+      e_r = sh.Srank[tid];
+      res = e_r >= a.res_first && e_r < a.res_first + a.res_count;
+    }
+    const unsigned bal = __ballot_sync(kFull, res);
+    if (lane == 0) sh.warp_tot[warp] = (unsigned long long)__popc(bal);
+    __syncthreads();                         // every thread has read its entry of sh.Srank
+    int pos = __popc(bal & ((1u << lane) - 1u));
+    for (int w = 0; w < warp; ++w) pos += (int)sh.warp_tot[w];
+    nS_l = 0;
+    for (int w = 0; w < n_warps; ++w) nS_l += (int)sh.warp_tot[w];
+    if (res) sh.Srank[pos] = e_r;
+    __syncthreads();
+  }
+  // publish the shortlist (unless the router kernel has): the FFN kernel's CTAs start streaming the weights of its best-ranked experts while
+  // the rest of the routing runs.  One word per rank (the expert, plus one; -1 beyond the last one): a CTA
+  // polls the word of the rank it starts on and needs nothing else, so each word is its own payload and a
+  // relaxed store suffices.
+  if (publish && tid < N)
+    asm volatile("st.relaxed.gpu.global.s32 [%0], %1;" ::"l"(ws.early_flag + tid), "r"(tid < nS_l ? sh.Srank[tid] + 1 : -1)
+                 : "memory");
+
+  return Shortlist{nS, nS_l, n_union};
+}
+
+// What remains once every token's kept experts are known: offsets, rows, work units and statistics, by one CTA.  kOneCta:
+// the kept experts lie in this CTA's shared memory (sh.colmask, one word per expert, and s_assign), else in the call's
+// accumulators, which are cleared for the next call.
+template <bool kOneCta>
+__device__ __forceinline__ void finish_call(const RouteArgs &a, RouteShared &sh, const Shortlist &sl, const short *s_assign) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n_warps = blockDim.x >> 5;
+  const int M = a.M, N = a.N, k = a.k;
+  const int mw = (a.M + 31) >> 5;     // words per expert row of the bit matrix in this call
+  const Workspace &ws = a.ws;
+  if (tid < N) sh.all_dense[tid] = 0;      // (set below, behind a barrier, for trees with early start)
+
+  // rows per expert and exclusive scans of rows, token chunks and active experts (Appendix C gather)
+  const int used_words = (M + 31) >> 5;
+  const bool cm_cached = N * used_words <= kColmaskCache;
+  {
+    const int c = tid >= N ? 0 : kOneCta ? __popc(sh.colmask[tid]) : __ldcg(ws.count_acc + tid);
+    if (!kOneCta && cm_cached)
+      for (int i = tid; i < N * used_words; i += blockDim.x) sh.colmask[i] = __ldcg(ws.colmask + i);
+    // work units and the active count cover the resident experts only; rows and offsets cover all
+    const bool resident = tid >= a.res_first && tid < a.res_first + a.res_count;
+    const int chunks = resident ? (c + a.chunk - 1) / a.chunk : 0;
+    // rows in bits 0..23, chunks in bits 24..43, active flag in bits 44..
+    const unsigned long long v = (unsigned long long)c | ((unsigned long long)chunks << 24) |
+                                 ((unsigned long long)(c > 0 && resident) << 44);
+    unsigned long long inc = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned long long up = __shfl_up_sync(kFull, inc, o);
+      if (lane >= o) inc += up;
+    }
+    if (lane == 31) sh.warp_tot[warp] = inc;
+    __syncthreads();
+    unsigned long long pre = inc - v;
+    for (int w = 0; w < warp; ++w) pre += sh.warp_tot[w];
+    if (tid < N) {
+      const int row0 = (int)(pre & 0xFFFFFFull), ub = (int)((pre >> 24) & 0xFFFFFull), ai = (int)(pre >> 44);
+      sh.count[tid] = c;
+      sh.offset[tid] = row0;
+      sh.unit_base[tid] = ub;
+      sh.cand[tid] = chunks;                // (the candidate flags are no longer needed: token chunks per expert)
+      ws.count[tid] = c;
+      ws.offset[tid] = row0;
+      ws.score[tid] = (double)sh.fx[tid] * (1.0 / kScoreScale);
+      if (c > 0 && resident) ws.active[ai] = tid;
+      for (int cc = 0; cc < chunks && ub + cc < 2 * kMaxExperts; ++cc) sh.chunk_expert[ub + cc] = tid;
+      if (tid == N - 1) {
+        sh.offset[N] = row0 + c;
+        ws.offset[N] = row0 + c;
+        sh.unit_base[N] = ub + chunks;
+        sh.nchunks = ub + chunks;
+        sh.nactive = ai + (c > 0 && resident);
+      }
+    }
+  }
+  __syncthreads();
+  if (a.early) {
+    // Early start (M <= 128, so an expert has at most one token chunk): the unit list follows the
+    // shortlist's rank order, and the experts whose gate/up units the FFN kernel's CTAs start on before
+    // this list exists (CTA c takes unit c) keep their place even if no token was routed to them.
+    // The gate/up units that CTAs may start on early (the first `ffn_ctas` of the list) are marked as taking
+    // all tokens from `hidden`, whoever draws them and when; an expert all of whose gate/up units are among
+    // them has no reader for its rows of the gathered copy, and they are not made.
+    const int n_head = min((a.ffn_ctas + a.tiles_up - 1) / a.tiles_up, sl.nS_l);
+    bool present = false;
+    int e_r = 0;
+    if (tid < sl.nS_l) {
+      e_r = sh.Srank[tid];
+      present = sh.count[e_r] > 0 || tid < n_head;
+      if ((tid + 1) * a.tiles_up <= a.ffn_ctas) sh.all_dense[e_r] = 1;
+    }
+    const unsigned bal = __ballot_sync(kFull, present);
+    if (lane == 0) sh.warp_tot[warp] = (unsigned long long)__popc(bal);
+    __syncthreads();
+    int pos = __popc(bal & ((1u << lane) - 1u));
+    for (int w = 0; w < warp; ++w) pos += (int)sh.warp_tot[w];
+    if (present) {
+      sh.unit_base[e_r] = pos;
+      sh.chunk_expert[pos] = e_r;
+    }
+    if (tid == 0) {
+      int tot = 0;
+      for (int w = 0; w < n_warps; ++w) tot += (int)sh.warp_tot[w];
+      sh.nchunks = tot;
+    }
+    __syncthreads();
+  } else if (a.tiles_up > 0 && (M <= 2 * kMaxTokChunk || a.rank_order)) {
+    // Trees of up to 256 tokens without early start: the listed experts in the shortlist's rank order too, each
+    // with its one or two token chunks.  Rank order is roughly row-count order, so the units that take longest
+    // (two full chunks, whose slabs are read twice) are handed out first and the list ends with cheap ones; in
+    // expert-index order whatever expert came last decided how long the CTAs waited for the last of them
+    // (-1 to -3 us at 129 to 255 tokens).  Larger trees on the one-SM kernel keep the index order of the scan
+    // above: with three and more chunks per popular expert, rank order bunches the units that live on L2
+    // re-reads at the start of the list, and the stream is slower there than with heavy and light experts
+    // interleaved (+2 % at 511 tokens, unbudgeted).  Calls that go to SM pairs ask for rank order whatever
+    // their size (rank_order): their units hold up to 256 rows, and the list ends with the small ones.
+    int e_r = 0, ch = 0;
+    if (tid < sl.nS_l) {
+      e_r = sh.Srank[tid];
+      ch = sh.cand[e_r];
+    }
+    int inc = ch;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int up = __shfl_up_sync(kFull, inc, o);
+      if (lane >= o) inc += up;
+    }
+    if (lane == 31) sh.warp_tot[warp] = (unsigned long long)inc;
+    __syncthreads();                       // (also: every thread is done with the index-order bases)
+    int pre = inc - ch;
+    for (int w = 0; w < warp; ++w) pre += (int)sh.warp_tot[w];
+    if (tid < sl.nS_l) {
+      sh.unit_base[e_r] = pre;
+      for (int cc = 0; cc < ch && pre + cc < 2 * kMaxExperts; ++cc) sh.chunk_expert[pre + cc] = e_r;
+    }
+    __syncthreads();
+  }
+
+  // The rest is three independent jobs, each latency-bound, run side by side:
+  //   warps 0-3  row of every (token, slot)       warps 4-6 (8-15)  work-unit list       warp 7  coverage
+  const int n_chunks = sh.nchunks;
+  double cov = 0.0;
+  if (warp < 4 && !a.rows_later) {
+    // rows ordered by (expert ascending, token ascending): the row of (t, e) is
+    // offset[e] + number of tokens below t that were also routed to e
+    // thread -> (token, slot) with the slot count padded to a power of two (no integer division)
+    int kshift = 0;
+    while ((1 << kshift) < k) ++kshift;
+    const int slot = tid & ((1 << kshift) - 1);
+    const int tok_step = 128 >> kshift;                    // tokens covered per pass by these 128 threads
+    for (int t0 = tid >> kshift; t0 < M; t0 += 4 * tok_step) {
+      int e[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int tt = t0 + u * tok_step;
+        e[u] = (tt < M && slot < k) ? __ldcg(ws.assign_idx + (size_t)tt * k + slot) : -1;
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int tt = t0 + u * tok_step;
+        if (tt >= M || slot >= k) continue;
+        int row = -1;
+        if (e[u] >= 0) {
+          const unsigned *cm = cm_cached ? sh.colmask + e[u] * used_words : ws.colmask + (size_t)e[u] * mw;
+          int below = 0;
+          if (cm_cached) {
+            below = __popc(cm[tt >> 5] & ((1u << (tt & 31)) - 1u));
+            for (int w = 0; w < (tt >> 5); ++w) below += __popc(cm[w]);
+          } else {
+            below = __popc(__ldcg(cm + (tt >> 5)) & ((1u << (tt & 31)) - 1u));
+            for (int w = 0; w < (tt >> 5); ++w) below += __popc(__ldcg(cm + w));
+          }
+          row = sh.offset[e[u]] + below;
+          ws.perm_row2tok[row] = tt;
+          ws.row2expert[row] = e[u];
+          if (ws.gather_src) ws.gather_src[row] = sh.all_dense[e[u]] ? -1 : tt;
+        }
+        ws.tokslot2row[(size_t)tt * k + slot] = row;
+      }
+    }
+  } else if (warp >= 4 && warp != 7) {
+    // work units (expert, token chunk, 128-row slab): all gate/up units, then all down
+    // units, each group ordered by (expert, chunk, slab); ready counters and the dispenser start at 0
+    if (a.tiles_up > 0) {
+      const int lt = warp < 7 ? tid - 128 : tid - 160, nthr = blockDim.x - 160;
+      const int n_up = n_chunks * a.tiles_up, n_down = n_chunks * a.tiles_down;
+      for (int i = lt; i < n_chunks; i += nthr) ws.ready[i] = 0;
+      for (int u = lt; u < n_up + n_down; u += nthr) {
+        const int phase = u >= n_up;
+        const int tiles = phase ? a.tiles_down : a.tiles_up;
+        const int v = phase ? u - n_up : u;
+        const int cpos = v / tiles;           // position in chunk-prefix space: identifies the expert
+        if (a.early) {                        // one chunk per listed expert, rank order
+          const int e1 = sh.chunk_expert[cpos];
+          ws.units[u] = Unit{e1, v - cpos * tiles, sh.offset[e1], sh.count[e1], cpos, phase,
+                             (!phase && (a.dense_all || u < a.ffn_ctas)) ? 2 : 0, 0};
+          continue;
+        }
+        int e;
+        if (cpos < 2 * kMaxExperts) {
+          e = sh.chunk_expert[cpos];
+        } else {          // more than 2N token chunks (M far beyond 128): search the chunk bases, in rank order
+          e = 0;
+          for (int r = 0; r < N; ++r) {          // (whatever the order of the list: the intervals are disjoint)
+            if (sh.cand[r] > 0 && sh.unit_base[r] <= cpos && cpos < sh.unit_base[r] + sh.cand[r]) { e = r; break; }
+          }
+        }
+        // inside an expert: slab-major, token chunk innermost, so the chunks that re-read a slab are
+        // handed out back to back and the second read hits L2
+        const int chunks_e = sh.cand[e];
+        const int local = v - sh.unit_base[e] * tiles;
+        const int tl = local / chunks_e, c = local - tl * chunks_e;
+        const int row0 = sh.offset[e] + c * a.chunk;
+        const int rows = min(a.chunk, sh.count[e] - c * a.chunk);
+        ws.units[u] = Unit{e, tl, row0, rows, sh.unit_base[e] + c, phase, (a.dense_all && !phase) ? 2 : 0, 0};
+      }
+    }
+  } else if (warp == 7) {
+    for (int e = lane; e < N; e += 32)
+      if ((sh.Smask[e >> 5] >> (e & 31)) & 1u) cov += (double)sh.fx[e];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) cov += shfl_xor_double(cov, o);
+    cov *= 1.0 / kScoreScale;
+  }
+  if (tid == 224) {         // lane 0 of warp 7, which holds the coverage sum
+    const int R = sh.offset[N];
+    ws.counters[0] = sl.nS;
+    ws.counters[1] = sh.nactive;
+    ws.counters[2] = R;
+    ws.counters[3] = n_chunks * a.tiles_up;
+    ws.counters[4] = n_chunks * a.tiles_down;
+    moespec_stats st;
+    st.n_union = sl.n_union;
+    st.n_shortlist = sl.nS;
+    st.n_active = sh.nactive;
+    st.n_rows = R;
+    st.n_dropped = M * k - R;
+    st.status = 0;
+    st.coverage = M > 0 ? cov / (double)M : 0.0;
+    st.weight_bytes = (long long)sh.nactive * a.expert_bytes;
+    *ws.stats = st;
+    *ws.status = 0;
+    if (!kOneCta) *ws.arrive_route = 0;
+  }
+  if (kOneCta) return;            // nothing of the call's accumulators was used
+  __syncthreads();
+  for (int i = tid; i < N; i += blockDim.x) {
+    ws.score_fx[i] = 0ull;
+    ws.natcnt_acc[i] = 0;
+    ws.count_acc[i] = 0;
+  }
+  // with rows_later the bit matrix is still needed by the row kernel and is cleared by the next call's
+  // first kernel instead
+  if (!a.rows_later)
+    for (int i = tid; i < N * used_words; i += blockDim.x) ws.colmask[i] = 0u;
 }
 
 // ---------------------------------------------------------------------------
@@ -695,31 +1081,18 @@ __device__ __forceinline__ void route_token(const RouteArgs &a, int t, int nS, c
 // ---------------------------------------------------------------------------
 template <int W>
 __global__ void __launch_bounds__(kRouteWarps * 32) route_kernel(RouteArgs a) {
-  __shared__ unsigned long long s_score[kMaxExperts];     // ranking key (score + 1, or 0 for a non-candidate)
-  __shared__ unsigned long long s_fx[kMaxExperts];        // fixed-point score
-  __shared__ unsigned s_colmask[kColmaskCache];
-  __shared__ int s_cand[kMaxExperts];
-  __shared__ int s_count[kMaxExperts];
-  __shared__ int s_offset[kMaxExperts + 1];
-  __shared__ int s_unit_base[kMaxExperts + 1];
-  __shared__ int s_Srank[kMaxExperts];
-  __shared__ uint32_t s_Smask[kMaskWords];
-  __shared__ unsigned long long s_warp_tot[kRouteWarps];
-  __shared__ int s_chunk_expert[kMaxExperts * 2];     // token chunk -> expert (first 2N chunks; more fall back)
-  __shared__ int s_nactive, s_last, s_nchunks;
-  __shared__ unsigned char s_all_dense[kMaxExperts];   // expert whose gate/up units all take every token from hidden
+  __shared__ RouteShared sh;
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int M = a.M, N = a.N, k = a.k;
-  const int mw = (a.M + 31) >> 5;     // words per expert row of the bit matrix in this call
   const Workspace &ws = a.ws;
   const int t = blockIdx.x * kRouteWarps + warp;
 
-  // With a router-based shortlist dependents are released only after the router kernel has completed:
+  // If this kernel publishes the shortlist, dependents are released only after the router kernel has completed:
   // the FFN kernel may then start while this kernel runs, and must find the shortlist flag already reset
-  // by the router kernel.  With a fixed shortlist (Eq. 4) the FFN kernel needs nothing from the router to
-  // begin streaming, so it is released at once.
-  if (a.early && a.shortlist == MOESPEC_STATIC) {
+  // by the router kernel.  With a fixed shortlist (Eq. 4), or one that the router kernel publishes, the FFN kernel needs
+  // nothing from here to begin streaming, so it is released at once.
+  if (a.early && (a.shortlist == MOESPEC_STATIC || a.from_router)) {
     pdl_trigger();
     pdl_wait();
   } else {
@@ -748,318 +1121,255 @@ __global__ void __launch_bounds__(kRouteWarps * 32) route_kernel(RouteArgs a) {
   if (tid < N) {
     const unsigned long long fx = __ldcg(ws.score_fx + tid);
     in_union = __ldcg(ws.natcnt_acc + tid) > 0;
-    s_cand[tid] = (a.shortlist == MOESPEC_FROM_UNION) ? in_union : 1;
-    s_score[tid] = s_cand[tid] ? fx + 1ull : 0ull;        // ranking key: candidates first, then by score
-    s_fx[tid] = fx;
+    sh.cand[tid] = (a.shortlist == MOESPEC_FROM_UNION) ? in_union : 1;
+    sh.score[tid] = sh.cand[tid] ? fx + 1ull : 0ull;        // ranking key: candidates first, then by score
+    sh.fx[tid] = fx;
   }
-  const int n_union = __syncthreads_count(in_union);
-  const int n_cand = __syncthreads_count(tid < N && s_cand[tid]);
-  const bool fixed = a.shortlist == MOESPEC_STATIC;
-  const int nS = fixed ? min(a.B, ws.n_static) : min(a.B, n_cand);
-  if (fixed) {
-    // static ranking (Eq. 4): the shortlist is the first nS experts of the fixed ordering
-    bool in_S = false;
-    if (tid < N) {
-      const int pos = ws.static_pos[tid];
-      in_S = pos < nS;
-      if (in_S) {
-        s_Srank[pos] = tid;
-        if (blockIdx.x == 0) ws.S_rank[pos] = tid;
-      }
-    }
-    const unsigned word = __ballot_sync(kFull, in_S);
-    if (lane == 0) s_Smask[warp] = word;
-  } else {
-    // one thread per expert; every thread walks the same j, so the shared-memory reads are broadcasts
-    // Branch-free rank by counting.  s_score holds score+1 for candidates and 0 for the others, so a
-    // non-candidate never outranks a candidate.
-    bool in_S = false;
-    if (tid < N) {
-      const unsigned long long si = s_score[tid];
-      int rank = 0;
-#pragma unroll 16
-      for (int j = 0; j < N; ++j) {
-        const unsigned long long sj = s_score[j];
-        rank += (int)((sj > si) | ((sj == si) & (j < tid)));
-      }
-      in_S = si != 0ull && rank < nS;
-      if (in_S) {
-        s_Srank[rank] = tid;
-        if (blockIdx.x == 0) ws.S_rank[rank] = tid;
-      }
-    }
-    const unsigned word = __ballot_sync(kFull, in_S);     // thread index = expert index: warp w owns mask word w
-    if (lane == 0) s_Smask[warp] = word;
-  }
-  __syncthreads();
-  // What the FFN kernel works on is the part of the shortlist that is resident on this GPU, in rank order
-  // (all of it unless this layer is an expert-parallel shard): s_Srank / nS_l from here on.  The shortlist
-  // itself stays in s_Smask (re-routing) and in ws.S_rank.
-  const bool shard = a.res_count < N;
-  int nS_l = nS;
-  if (shard) {
-    int e_r = 0;
-    bool res = false;
-    if (tid < nS) {
-      e_r = s_Srank[tid];
-      res = e_r >= a.res_first && e_r < a.res_first + a.res_count;
-    }
-    const unsigned bal = __ballot_sync(kFull, res);
-    if (lane == 0) s_warp_tot[warp] = (unsigned long long)__popc(bal);
-    __syncthreads();                         // every thread has read its entry of s_Srank
-    int pos = __popc(bal & ((1u << lane) - 1u));
-    for (int w = 0; w < warp; ++w) pos += (int)s_warp_tot[w];
-    nS_l = 0;
-    for (int w = 0; w < kRouteWarps; ++w) nS_l += (int)s_warp_tot[w];
-    if (res) s_Srank[pos] = e_r;
-    __syncthreads();
-  }
-  // publish the shortlist: the FFN kernel's CTAs start streaming the weights of its best-ranked experts while
-  // the rest of the routing runs.  One word per rank (the expert, plus one; -1 beyond the last one): a CTA
-  // polls the word of the rank it starts on and needs nothing else, so each word is its own payload and a
-  // relaxed store suffices.
-  if (blockIdx.x == 0 && ws.early_flag && tid < N)
-    asm volatile("st.relaxed.gpu.global.s32 [%0], %1;" ::"l"(ws.early_flag + tid), "r"(tid < nS_l ? s_Srank[tid] + 1 : -1)
-                 : "memory");
+  const Shortlist sl = pick_shortlist<kMaxExperts>(a, sh, in_union, blockIdx.x == 0, blockIdx.x == 0 && ws.early_flag && !a.from_router);
 
   // ---- re-routing (Eq. 7 / Eq. 8) and mixing weights (Section 3.3) of this warp's token
-  if (t < M) route_token<W>(a, t, nS, s_Smask, key, p, nat, lane);
+  if (t < M) token_reroute<W>(a, t, sl.nS, sh.Smask, key, p, nat, lane);
 
   // ---- the CTA that arrives last finishes the call
   __syncthreads();
   if (tid == 0) {
     const int prev = arrive_acq_rel(ws.arrive_route);
-    s_last = (prev == (int)gridDim.x - 1);
+    sh.last = (prev == (int)gridDim.x - 1);
   }
   __syncthreads();
-  if (!s_last) return;
-  if (tid < N) s_all_dense[tid] = 0;      // (set below, behind a barrier, for trees with early start)
-
-  // rows per expert and exclusive scans of rows, token chunks and active experts (Appendix C gather)
-  const int used_words = (M + 31) >> 5;
-  const bool cm_cached = N * used_words <= kColmaskCache;
-  {
-    const int c = tid < N ? __ldcg(ws.count_acc + tid) : 0;
-    if (cm_cached)
-      for (int i = tid; i < N * used_words; i += blockDim.x) s_colmask[i] = __ldcg(ws.colmask + i);
-    // work units and the active count cover the resident experts only; rows and offsets cover all
-    const bool resident = tid >= a.res_first && tid < a.res_first + a.res_count;
-    const int chunks = resident ? (c + a.chunk - 1) / a.chunk : 0;
-    // rows in bits 0..23, chunks in bits 24..43, active flag in bits 44..
-    const unsigned long long v = (unsigned long long)c | ((unsigned long long)chunks << 24) |
-                                 ((unsigned long long)(c > 0 && resident) << 44);
-    unsigned long long inc = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned long long up = __shfl_up_sync(kFull, inc, o);
-      if (lane >= o) inc += up;
-    }
-    if (lane == 31) s_warp_tot[warp] = inc;
-    __syncthreads();
-    unsigned long long pre = inc - v;
-    for (int w = 0; w < warp; ++w) pre += s_warp_tot[w];
-    if (tid < N) {
-      const int row0 = (int)(pre & 0xFFFFFFull), ub = (int)((pre >> 24) & 0xFFFFFull), ai = (int)(pre >> 44);
-      s_count[tid] = c;
-      s_offset[tid] = row0;
-      s_unit_base[tid] = ub;
-      s_cand[tid] = chunks;                // (the candidate flags are no longer needed: token chunks per expert)
-      ws.count[tid] = c;
-      ws.offset[tid] = row0;
-      ws.score[tid] = (double)s_fx[tid] * (1.0 / kScoreScale);
-      if (c > 0 && resident) ws.active[ai] = tid;
-      for (int cc = 0; cc < chunks && ub + cc < 2 * kMaxExperts; ++cc) s_chunk_expert[ub + cc] = tid;
-      if (tid == N - 1) {
-        s_offset[N] = row0 + c;
-        ws.offset[N] = row0 + c;
-        s_unit_base[N] = ub + chunks;
-        s_nchunks = ub + chunks;
-        s_nactive = ai + (c > 0 && resident);
-      }
-    }
-  }
-  __syncthreads();
-  if (a.early) {
-    // Early start (M <= 128, so an expert has at most one token chunk): the unit list follows the
-    // shortlist's rank order, and the experts whose gate/up units the FFN kernel's CTAs start on before
-    // this list exists (CTA c takes unit c) keep their place even if no token was routed to them.
-    // The gate/up units that CTAs may start on early (the first `ffn_ctas` of the list) are marked as taking
-    // all tokens from `hidden`, whoever draws them and when; an expert all of whose gate/up units are among
-    // them has no reader for its rows of the gathered copy, and they are not made.
-    const int n_head = min((a.ffn_ctas + a.tiles_up - 1) / a.tiles_up, nS_l);
-    bool present = false;
-    int e_r = 0;
-    if (tid < nS_l) {
-      e_r = s_Srank[tid];
-      present = s_count[e_r] > 0 || tid < n_head;
-      if ((tid + 1) * a.tiles_up <= a.ffn_ctas) s_all_dense[e_r] = 1;
-    }
-    const unsigned bal = __ballot_sync(kFull, present);
-    if (lane == 0) s_warp_tot[warp] = (unsigned long long)__popc(bal);
-    __syncthreads();
-    int pos = __popc(bal & ((1u << lane) - 1u));
-    for (int w = 0; w < warp; ++w) pos += (int)s_warp_tot[w];
-    if (present) {
-      s_unit_base[e_r] = pos;
-      s_chunk_expert[pos] = e_r;
-    }
-    if (tid == 0) {
-      int tot = 0;
-      for (int w = 0; w < kRouteWarps; ++w) tot += (int)s_warp_tot[w];
-      s_nchunks = tot;
-    }
-    __syncthreads();
-  } else if (a.tiles_up > 0 && (M <= 2 * kMaxTokChunk || a.rank_order)) {
-    // Trees of up to 256 tokens without early start: the listed experts in the shortlist's rank order too, each
-    // with its one or two token chunks.  Rank order is roughly row-count order, so the units that take longest
-    // (two full chunks, whose slabs are read twice) are handed out first and the list ends with cheap ones; in
-    // expert-index order whatever expert came last decided how long the CTAs waited for the last of them
-    // (-1 to -3 us at 129 to 255 tokens).  Larger trees on the one-SM kernel keep the index order of the scan
-    // above: with three and more chunks per popular expert, rank order bunches the units that live on L2
-    // re-reads at the start of the list, and the stream is slower there than with heavy and light experts
-    // interleaved (+2 % at 511 tokens, unbudgeted).  Calls that go to SM pairs ask for rank order whatever
-    // their size (rank_order): their units hold up to 256 rows, and the list ends with the small ones.
-    int e_r = 0, ch = 0;
-    if (tid < nS_l) {
-      e_r = s_Srank[tid];
-      ch = s_cand[e_r];
-    }
-    int inc = ch;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int up = __shfl_up_sync(kFull, inc, o);
-      if (lane >= o) inc += up;
-    }
-    if (lane == 31) s_warp_tot[warp] = (unsigned long long)inc;
-    __syncthreads();                       // (also: every thread is done with the index-order bases)
-    int pre = inc - ch;
-    for (int w = 0; w < warp; ++w) pre += (int)s_warp_tot[w];
-    if (tid < nS_l) {
-      s_unit_base[e_r] = pre;
-      for (int cc = 0; cc < ch && pre + cc < 2 * kMaxExperts; ++cc) s_chunk_expert[pre + cc] = e_r;
-    }
-    __syncthreads();
-  }
-
-  // The rest is three independent jobs, each latency-bound, run side by side:
-  //   warps 0-3  row of every (token, slot)       warps 4-6  work-unit list       warp 7  coverage
-  const int n_chunks = s_nchunks;
-  double cov = 0.0;
-  if (warp < 4 && !a.rows_later) {
-    // rows ordered by (expert ascending, token ascending): the row of (t, e) is
-    // offset[e] + number of tokens below t that were also routed to e
-    // thread -> (token, slot) with the slot count padded to a power of two (no integer division)
-    int kshift = 0;
-    while ((1 << kshift) < k) ++kshift;
-    const int slot = tid & ((1 << kshift) - 1);
-    const int tok_step = 128 >> kshift;                    // tokens covered per pass by these 128 threads
-    for (int t0 = tid >> kshift; t0 < M; t0 += 4 * tok_step) {
-      int e[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int tt = t0 + u * tok_step;
-        e[u] = (tt < M && slot < k) ? __ldcg(ws.assign_idx + (size_t)tt * k + slot) : -1;
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int tt = t0 + u * tok_step;
-        if (tt >= M || slot >= k) continue;
-        int row = -1;
-        if (e[u] >= 0) {
-          const unsigned *cm = cm_cached ? s_colmask + e[u] * used_words : ws.colmask + (size_t)e[u] * mw;
-          int below = 0;
-          if (cm_cached) {
-            below = __popc(cm[tt >> 5] & ((1u << (tt & 31)) - 1u));
-            for (int w = 0; w < (tt >> 5); ++w) below += __popc(cm[w]);
-          } else {
-            below = __popc(__ldcg(cm + (tt >> 5)) & ((1u << (tt & 31)) - 1u));
-            for (int w = 0; w < (tt >> 5); ++w) below += __popc(__ldcg(cm + w));
-          }
-          row = s_offset[e[u]] + below;
-          ws.perm_row2tok[row] = tt;
-          ws.row2expert[row] = e[u];
-          if (ws.gather_src) ws.gather_src[row] = s_all_dense[e[u]] ? -1 : tt;
-        }
-        ws.tokslot2row[(size_t)tt * k + slot] = row;
-      }
-    }
-  } else if (warp >= 4 && warp < 7) {
-    // work units (expert, token chunk, 128-row slab): all gate/up units, then all down
-    // units, each group ordered by (expert, chunk, slab); ready counters and the dispenser start at 0
-    if (a.tiles_up > 0) {
-      const int lt = tid - 128, nthr = 96;
-      const int n_up = n_chunks * a.tiles_up, n_down = n_chunks * a.tiles_down;
-      for (int i = lt; i < n_chunks; i += nthr) ws.ready[i] = 0;
-      for (int u = lt; u < n_up + n_down; u += nthr) {
-        const int phase = u >= n_up;
-        const int tiles = phase ? a.tiles_down : a.tiles_up;
-        const int v = phase ? u - n_up : u;
-        const int cpos = v / tiles;           // position in chunk-prefix space: identifies the expert
-        if (a.early) {                        // one chunk per listed expert, rank order
-          const int e1 = s_chunk_expert[cpos];
-          ws.units[u] = Unit{e1, v - cpos * tiles, s_offset[e1], s_count[e1], cpos, phase,
-                             (!phase && (a.dense_all || u < a.ffn_ctas)) ? 2 : 0, 0};
-          continue;
-        }
-        int e;
-        if (cpos < 2 * kMaxExperts) {
-          e = s_chunk_expert[cpos];
-        } else {          // more than 2N token chunks (M far beyond 128): search the chunk bases, in rank order
-          e = 0;
-          for (int r = 0; r < N; ++r) {          // (whatever the order of the list: the intervals are disjoint)
-            if (s_cand[r] > 0 && s_unit_base[r] <= cpos && cpos < s_unit_base[r] + s_cand[r]) { e = r; break; }
-          }
-        }
-        // inside an expert: slab-major, token chunk innermost, so the chunks that re-read a slab are
-        // handed out back to back and the second read hits L2
-        const int chunks_e = s_cand[e];
-        const int local = v - s_unit_base[e] * tiles;
-        const int tl = local / chunks_e, c = local - tl * chunks_e;
-        const int row0 = s_offset[e] + c * a.chunk;
-        const int rows = min(a.chunk, s_count[e] - c * a.chunk);
-        ws.units[u] = Unit{e, tl, row0, rows, s_unit_base[e] + c, phase, (a.dense_all && !phase) ? 2 : 0, 0};
-      }
-    }
-  } else if (warp == 7) {
-    for (int e = lane; e < N; e += 32)
-      if ((s_Smask[e >> 5] >> (e & 31)) & 1u) cov += (double)s_fx[e];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) cov += shfl_xor_double(cov, o);
-    cov *= 1.0 / kScoreScale;
-  }
-  if (tid == 224) {         // lane 0 of warp 7, which holds the coverage sum
-    const int R = s_offset[N];
-    ws.counters[0] = nS;
-    ws.counters[1] = s_nactive;
-    ws.counters[2] = R;
-    ws.counters[3] = n_chunks * a.tiles_up;
-    ws.counters[4] = n_chunks * a.tiles_down;
-    moespec_stats st;
-    st.n_union = n_union;
-    st.n_shortlist = nS;
-    st.n_active = s_nactive;
-    st.n_rows = R;
-    st.n_dropped = M * k - R;
-    st.status = 0;
-    st.coverage = M > 0 ? cov / (double)M : 0.0;
-    st.weight_bytes = (long long)s_nactive * a.expert_bytes;
-    *ws.stats = st;
-    *ws.status = 0;
-    *ws.arrive_route = 0;
-  }
-  __syncthreads();
-  for (int i = tid; i < N; i += blockDim.x) {
-    ws.score_fx[i] = 0ull;
-    ws.natcnt_acc[i] = 0;
-    ws.count_acc[i] = 0;
-  }
-  // with rows_later the bit matrix is still needed by the row kernel and is cleared by the next call's
-  // first kernel instead
-  if (!a.rows_later)
-    for (int i = tid; i < N * used_words; i += blockDim.x) ws.colmask[i] = 0u;
+  if (!sh.last) return;
+  finish_call<false>(a, sh, sl, nullptr);
 }
 
-static cudaError_t launch_route_kernel(const LaunchCtx &c, const float *logits) {
+// Shortlist from the completed scores and union, by one CTA, for the FFN kernel's CTAs that wait for it: as
+// pick_shortlist, but nothing is kept.
+__device__ __forceinline__ void publish_shortlist(const RouteArgs &a, unsigned long long *s_score) {
+  const int tid = threadIdx.x, N = a.N;
+  int gs = 0;
+  while ((N << (gs + 1)) <= (int)blockDim.x && gs < 3) ++gs;
+  const int i = tid >> gs, sub = tid & ((1 << gs) - 1);
+  if (tid < N) {
+    const unsigned long long fx = __ldcg(a.ws.score_fx + tid);
+    const bool cand = a.shortlist != MOESPEC_FROM_UNION || __ldcg(a.ws.natcnt_acc + tid) > 0;
+    s_score[tid] = cand ? fx + 1ull : 0ull;        // ranking key: candidates first, then by score
+  }
+  __syncthreads();
+  // 2^gs threads share an expert, each counts every 2^gs-th of those that outrank it: all of them, and the resident ones
+  const unsigned long long si = i < N ? s_score[i] : 0ull;
+  int rank = 0, rank_l = 0;
+  if (i < N) {
+#pragma unroll 4
+    for (int j = sub; j < N; j += 1 << gs) {
+      const unsigned long long sj = s_score[j];
+      const int over = (int)((sj > si) | ((sj == si) & (j < i)));
+      rank += over;
+      rank_l += over & (int)((unsigned)(j - a.res_first) < (unsigned)a.res_count);
+    }
+  }
+  for (int o = 1; o < (1 << gs); o <<= 1) {
+    rank += __shfl_xor_sync(kFull, rank, o);
+    rank_l += __shfl_xor_sync(kFull, rank_l, o);
+  }
+  const bool listed = i < N && sub == 0 && si != 0ull && rank < a.B && (unsigned)(i - a.res_first) < (unsigned)a.res_count;
+  // One word per rank (the expert, plus one; -1 beyond the last one): a CTA polls the word of the rank it starts on and
+  // needs nothing else, so each word is its own payload and a relaxed store suffices.
+  auto word = [&](int r, int v) {
+    asm volatile("st.relaxed.gpu.global.s32 [%0], %1;" ::"l"(a.ws.early_flag + r), "r"(v) : "memory");
+  };
+  if (listed) word(rank_l, i + 1);
+  const int n = __syncthreads_count(listed);
+  if (tid >= n && tid < N) word(tid, -1);
+}
+
+// ---------------------------------------------------------------------------
+// K1 for trees of up to 128 tokens and up to 128 experts: logits, softmax, top-k and scores, and for the FFN kernel's
+// early start the shortlist.  It is a chain of dependent steps in front of the weight stream, so what counts is how
+// long each takes, not how much work it is.  us from the return of its dependency wait, 63 tokens, 64 experts,
+// d = 2048: logits 0.9, exchange 1.75, softmax and top-k 3.4, last arrival 4.5, shortlist published 5.9 (the chain of
+// the router above and route_kernel published it 11 us after; a layer of 63 tokens, B = 32, 77.5 -> 74.7, one of 16
+// 72.5 -> 69.9).
+//   * A cluster of CTAs takes a token tile, each CTA 16 experts of it; the logits of a token meet in the shared memory
+//     of the CTA that owns the token (cluster_sync) instead of global memory and an arrival counter.
+//   * 16-bit layers: 16 experts x 8 tokens a CTA on mma.sync, K split over eight warps, every load of a batch issued
+//     before the first MMA and none behind a branch of its own (guarded loads were waited for one by one: 3300 cycles
+//     instead of 1100).  fp32 layers, and widths that do not split: 16 experts x 2 tokens on the CUDA cores, the sums of
+//     router_topk_kernel.
+//   * 8 warps of at most 136 registers and 5 KB of shared memory fit beside a CTA of the previous call's FFN kernel (10
+//     warps of 80), register file quarter by quarter, so that the CTAs are resident with their router rows loaded when
+//     that kernel ends.
+//   * The FFN kernel is released by this kernel's CTAs (through route_kernel and the gather, which release at once) and
+//     is resident when the shortlist comes.  Its control words have been reset by then: by a cluster of its own, whose
+//     release follows a fence.
+//   * The last CTA to arrive publishes the shortlist; route_kernel finds it again from the same scores.
+// ---------------------------------------------------------------------------
+constexpr int kTreeWarps = 8, kTreeExperts = 16, kTreeMaxN = 128;
+template <bool kMma> constexpr int kTreeTokens = kMma ? 8 : 2;      // token tile of a cluster
+
+template <typename T, bool kMma>
+__global__ void __maxnreg__(136) tree_router_kernel(const T *__restrict__ hidden, const T *__restrict__ Wr,
+                                                    const float *__restrict__ bias, int d, int publish, RouteArgs a) {
+  constexpr int TOK = kTreeTokens<kMma>;
+  __shared__ union {
+    float part[kTreeWarps][kTreeExperts * TOK];      // partial dot products of the warps
+    unsigned long long score[kTreeMaxN];
+  } sh;
+  __shared__ float s_z[kTreeMaxN];                        // logits of this CTA's tokens, N per token
+  __shared__ int s_last;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int M = a.M, N = a.N, k = a.k;
+  const Workspace &ws = a.ws;
+  const uint32_t C = gridDim.x;                       // CTAs of a cluster: the experts of one token tile
+  if (blockIdx.y == gridDim.y - 1) {                  // a cluster of its own prepares the FFN kernel's control words
+    pdl_wait();
+    if (blockIdx.x == 0) reset_ffn_control(ws.early_flag, N, ws.unit_counter, 1);
+    pdl_trigger();
+    for (int i = (int)blockIdx.x * blockDim.x + tid; i < N * ((M + 31) >> 5); i += C * blockDim.x) ws.colmask[i] = 0u;
+    return;
+  }
+  const uint32_t rank = blockIdx.x;
+  const int e0 = (int)rank * kTreeExperts, t0 = (int)blockIdx.y * TOK;
+  // C is a power of two
+  const int c_bits = 31 - __clz(C), slots = (TOK + (int)C - 1) >> c_bits;      // tokens of this CTA
+
+  constexpr int VEC = 16 / sizeof(T), U = kMma ? 8 : 4;
+  const int g = lane >> 2, tg = lane & 3, kw = d / kTreeWarps;      // kMma: K range of this warp
+  // two router rows of this thread (kMma) or warp; a constant of the layer, so their start is fetched before the wait
+  const T *w0 = Wr + (kMma ? (size_t)min(e0 + g, N - 1) * d + warp * kw + tg * 8 : (size_t)min(e0 + warp, N - 1) * d + lane * VEC);
+  const T *w1 = Wr + (kMma ? (size_t)min(e0 + g + 8, N - 1) * d + warp * kw + tg * 8
+                           : (size_t)min(e0 + warp + kTreeWarps, N - 1) * d + lane * VEC);
+  // the bias of the logits this thread will finish (kMma: one; else lane 0 of a warp two)
+  auto bias_of = [&](int e) { return bias && e < N ? load_early(bias + e) : 0.f; };
+  const float b0 = bias_of(kMma ? e0 + tid / TOK % kTreeExperts : e0 + warp);
+  const float b1 = kMma ? 0.f : bias_of(e0 + warp + kTreeWarps);
+  uint4 W0[8], W1[8];
+#pragma unroll
+  for (int s = 0; s < 8; ++s)
+    if (kMma || (lane + s * 32) * VEC < d) {
+      const int off = kMma ? (s * 32 < kw ? s * 32 : 0) : s * 32 * VEC;
+      W0[s] = load_early((const void *)(w0 + off));
+      W1[s] = load_early((const void *)(w1 + off));
+    }
+  // ... and so are the kernel's arguments, whose lines of the constant bank each cost a miss at their first use
+  const T *hb = hidden + (kMma ? (size_t)min(t0 + g, M - 1) * d + warp * kw + tg * 8 : (size_t)0);
+  asm volatile("" ::"l"(hb), "l"(ws.logits), "l"(ws.prob), "l"(ws.score_fx), "l"(ws.topk_idx), "l"(ws.natcnt_acc), "l"(ws.arrive),
+               "l"(ws.early_flag), "r"(M), "r"(N), "r"(k), "r"(a.B), "r"(a.shortlist), "r"(a.res_first), "r"(publish));
+  cluster_sync();        // the CTAs of the cluster have started
+  pdl_wait();
+  pdl_trigger();
+  // a finished logit goes to the CTA of the cluster that owns its token
+  auto finish_logit = [&](int tl, int e, float z) {
+    if (e >= N || t0 + tl >= M) return;
+    st_cluster(&s_z[(tl >> c_bits) * N + e], tl & (C - 1), __float_as_uint(z));
+    ws.logits[(size_t)(t0 + tl) * N + e] = z;
+  };
+  if constexpr (kMma) {
+    float c[4] = {0.f, 0.f, 0.f, 0.f};
+    // `steps` times 32 elements of K from k0 on; all loads are issued before the first MMA
+    auto block = [&](auto reload, int k0, int steps) {
+      uint4 X[U];
+#pragma unroll
+      for (int s = 0; s < U; ++s) {
+        const int off = k0 + (s < steps ? s : 0) * 32;        // (steps is U, or the remainder: those repeat the first)
+        X[s] = *reinterpret_cast<const uint4 *>(hb + off);
+        if constexpr (decltype(reload)::value) {
+          W0[s] = *reinterpret_cast<const uint4 *>(w0 + off);
+          W1[s] = *reinterpret_cast<const uint4 *>(w1 + off);
+        }
+      }
+      // Every MMA starts from zero and the running sums are kept in fp32 registers: a chain of MMAs on one accumulator
+      // rounds worse than the CUDA-core dot product.
+#pragma unroll
+      for (int s = 0; s < U; ++s) {
+        float lo[4] = {0.f, 0.f, 0.f, 0.f}, hi[4] = {0.f, 0.f, 0.f, 0.f};
+        mma_16816(lo, W0[s].x, W1[s].x, W0[s].y, W1[s].y, X[s].x, X[s].y, T());
+        mma_16816(hi, W0[s].z, W1[s].z, W0[s].w, W1[s].w, X[s].z, X[s].w, T());
+#pragma unroll
+        for (int q = 0; q < 4; ++q) c[q] += s < steps ? lo[q] + hi[q] : 0.f;
+      }
+    };
+    block(std::false_type(), 0, min(U, kw / 32));
+    for (int k0 = 32 * U; k0 < kw; k0 += 32 * U) block(std::true_type(), k0, min(U, (kw - k0) / 32));
+    float2 *part = reinterpret_cast<float2 *>(&sh.part[warp][g * TOK + 2 * tg]);
+    part[0] = make_float2(c[0], c[1]);
+    part[4 * TOK] = make_float2(c[2], c[3]);
+    __syncthreads();
+    if (tid < kTreeExperts * TOK) {
+      float v[kTreeWarps];
+#pragma unroll
+      for (int w = 0; w < kTreeWarps; ++w) v[w] = sh.part[w][tid];
+#pragma unroll
+      for (int o = 1; o < kTreeWarps; o <<= 1)
+#pragma unroll
+        for (int w = 0; w < kTreeWarps; w += 2 * o) v[w] += v[w + o];
+      finish_logit(tid % TOK, e0 + tid / TOK, v[0] + b0);
+    }
+  } else {
+    float acc[2][TOK] = {};
+    for (int j0 = lane * VEC; j0 < d; j0 += 64 * VEC * U) {
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int jh = j0 + h * 32 * VEC * U;
+        if (j0 != lane * VEC) {
+#pragma unroll
+          for (int u = 0; u < U; ++u)
+            if (jh + u * 32 * VEC < d) {
+              W0[h * U + u] = *reinterpret_cast<const uint4 *>(w0 + jh - lane * VEC + u * 32 * VEC);
+              W1[h * U + u] = *reinterpret_cast<const uint4 *>(w1 + jh - lane * VEC + u * 32 * VEC);
+            }
+        }
+#pragma unroll
+        for (int tt = 0; tt < TOK; ++tt) {
+          const T *hr = hidden + (size_t)min(t0 + tt, M - 1) * d;      // clamp: a token beyond M repeats the last row
+          uint4 X[U];
+#pragma unroll
+          for (int u = 0; u < U; ++u)
+            if (jh + u * 32 * VEC < d) X[u] = *reinterpret_cast<const uint4 *>(hr + jh + u * 32 * VEC);
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            if (jh + u * 32 * VEC < d) {
+              const T *ew0 = reinterpret_cast<const T *>(&W0[h * U + u]), *ew1 = reinterpret_cast<const T *>(&W1[h * U + u]);
+              const T *eh = reinterpret_cast<const T *>(&X[u]);
+#pragma unroll
+              for (int v = 0; v < VEC; ++v) {
+                acc[0][tt] = fmaf(to_float(ew0[v]), to_float(eh[v]), acc[0][tt]);
+                acc[1][tt] = fmaf(to_float(ew1[v]), to_float(eh[v]), acc[1][tt]);
+              }
+            }
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int tt = 0; tt < TOK; ++tt) {
+        float z = acc[h][tt];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(kFull, z, o);
+        if (lane == 0) finish_logit(tt, e0 + warp + h * kTreeWarps, z + (h ? b1 : b0));
+      }
+  }
+  cluster_sync();              // slot q of this CTA is token t0 + q * C + rank
+  // softmax (Eq. 1), scores (Eq. 5), natural top-k (Eq. 2) and union (Eq. 3): two warps per token
+  for (int item = warp; item < 2 * slots; item += kTreeWarps) {
+    const int q = item >> 1, tl = q * (int)C + (int)rank, t = t0 + tl;
+    if (tl < TOK && t < M)
+      token_phase(s_z + q * N, N, k, ws.prob + (size_t)t * N, ws.topk_idx + (size_t)t * k, ws.score_fx, ws.natcnt_acc, lane,
+                  1 + (item & 1));
+  }
+  if (!publish) return;
+  // the CTA that arrives last knows every score: it publishes the shortlist
+  __syncthreads();
+  if (tid == 0) {
+    const int n = (int)(gridDim.x * (gridDim.y - 1));
+    s_last = arrive_acq_rel(ws.arrive) == n - 1;
+    if (s_last) ws.arrive[0] = 0;
+  }
+  __syncthreads();
+  if (s_last) publish_shortlist(a, sh.score);
+}
+
+static RouteArgs route_args(const LaunchCtx &c, const float *logits) {
   const moespec_layer_desc &D = *c.desc;
   RouteArgs a;
   a.logits = logits;
@@ -1074,14 +1384,46 @@ static cudaError_t launch_route_kernel(const LaunchCtx &c, const float *logits) 
   a.rows_later = rows_in_row_kernel(c.M);
   a.chunk = c.chunk;
   a.rank_order = c.rank_order;
+  a.from_router = c.ru > 0 && c.early && D.shortlist != MOESPEC_STATIC && tree_router_takes(c);
   a.dense_all = c.ru > 0 ? c.dense_all : 0;
   a.res_first = c.res_count > 0 ? c.res_first : 0;
   a.res_count = c.res_count > 0 ? c.res_count : D.n_experts;
+  return a;
+}
+
+static cudaError_t launch_route_kernel(const LaunchCtx &c, const float *logits) {
+  const RouteArgs a = route_args(c, logits);
   const dim3 grid((c.M + kRouteWarps - 1) / kRouteWarps), block(kRouteWarps * 32);
   if (a.N <= 32) return launch_kernel(route_kernel<1>, grid, block, 0, c.stream, a);
   if (a.N <= 64) return launch_kernel(route_kernel<2>, grid, block, 0, c.stream, a);
   if (a.N <= 128) return launch_kernel(route_kernel<4>, grid, block, 0, c.stream, a);
   return launch_kernel(route_kernel<8>, grid, block, 0, c.stream, a);
+}
+
+static bool tree_router_takes(const LaunchCtx &c) { return c.M <= kMaxTokChunk && c.desc->n_experts <= kTreeMaxN; }
+
+template <typename T, bool kMma>
+static cudaError_t launch_tree_router_t(const LaunchCtx &c, const void *hidden) {
+  const moespec_layer_desc &D = *c.desc;
+  RouteArgs a = route_args(c, c.ws->logits);
+  int C = 1;
+  while (C * kTreeExperts < D.n_experts) C *= 2;
+  const int tiles = (c.M + kTreeTokens<kMma> - 1) / kTreeTokens<kMma>;
+  return launch_kernel_cluster(tree_router_kernel<T, kMma>, dim3(C, tiles + 1), dim3(kTreeWarps * 32), C, c.stream,
+                               (const T *)hidden, (const T *)D.router_w, D.router_bias, D.d, a.from_router, a);
+}
+
+template <typename T>
+static cudaError_t launch_tree_router(const LaunchCtx &c, const void *hidden) {
+  if constexpr (sizeof(T) == 2)
+    if (c.desc->d % (32 * kTreeWarps) == 0) return launch_tree_router_t<T, true>(c, hidden);
+  return launch_tree_router_t<T, false>(c, hidden);
+}
+
+static cudaError_t launch_router_for_tree(const LaunchCtx &c, const void *hidden) {
+  if (c.desc->dtype == MOESPEC_BF16) return launch_tree_router<__nv_bfloat16>(c, hidden);
+  if (c.desc->dtype == MOESPEC_FP16) return launch_tree_router<__half>(c, hidden);
+  return launch_tree_router<float>(c, hidden);
 }
 
 // Eq. 4: add the natural top-k counts of the last router launch to the calibration counters and
@@ -1236,6 +1578,11 @@ cudaError_t routing_configure() {
   set((const void *)route_kernel<2>);
   set((const void *)route_kernel<4>);
   set((const void *)route_kernel<8>);
+  set((const void *)tree_router_kernel<__nv_bfloat16, true>);
+  set((const void *)tree_router_kernel<__half, true>);
+  set((const void *)tree_router_kernel<__nv_bfloat16, false>);
+  set((const void *)tree_router_kernel<__half, false>);
+  set((const void *)tree_router_kernel<float, false>);
   set((const void *)gather_rows_kernel);
   set((const void *)rows_gather_kernel);
   return e;
