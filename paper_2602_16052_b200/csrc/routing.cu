@@ -327,7 +327,7 @@ __global__ void __launch_bounds__(256) router_topk_kernel(const T *__restrict__ 
 }
 
 // ---------------------------------------------------------------------------
-// K1 for larger trees: the same logits, softmax and top-k, with the dot products on the tensor cores.
+// K1 for larger trees and wide routers: the same logits, softmax and top-k, with the dot products on the tensor cores.
 // A CTA takes 16 experts x 8 tokens; its NW (sixteen, or eight) warps split K, each running m16n8k16 MMAs (experts on the
 // M axis, tokens on the N axis) on operands loaded straight from global memory: thread (g, tg) of a warp
 // reads 16 contiguous bytes of router rows g and g+8 and of token row g at K offset 32*step + 8*tg and
@@ -523,8 +523,8 @@ cudaError_t launch_router_mma<float, 8>(const LaunchCtx &, const void *) { retur
 template <>
 cudaError_t launch_router_mma<float, 16>(const LaunchCtx &, const void *) { return cudaErrorNotSupported; }
 
-// Trees beyond 64 tokens of a 16-bit layer take the tensor-core router (d must split into eight K ranges of
-// whole 32-element steps).
+// Trees beyond 64 tokens of a 16-bit layer that tree_router_kernel does not take have their products on the tensor cores
+// all the same (d must split into eight K ranges of whole 32-element steps).
 static bool use_router_mma(const LaunchCtx &c) {
   static const bool off = [] { const char *v = experiment_env("MOESPEC_NO_ROUTER_MMA"); return v && v[0] == '1'; }();
   static const int min_m = [] { const char *v = experiment_env("MOESPEC_ROUTER_MMA_MIN_M"); return v ? atoi(v) : 65; }();
@@ -1182,7 +1182,7 @@ __device__ __forceinline__ void publish_shortlist(const RouteArgs &a, unsigned l
 }
 
 // ---------------------------------------------------------------------------
-// K1 for trees of up to 128 tokens and up to 128 experts: logits, softmax, top-k and scores, and for the FFN kernel's
+// K1 for small trees (tree_router_takes) and up to 128 experts: logits, softmax, top-k and scores, and for the FFN kernel's
 // early start the shortlist.  It is a chain of dependent steps in front of the weight stream, so what counts is how
 // long each takes, not how much work it is.  us from the return of its dependency wait, 63 tokens, 64 experts,
 // d = 2048: logits 0.9, exchange 1.75, softmax and top-k 3.4, last arrival 4.5, shortlist published 5.9 (the chain of
@@ -1400,7 +1400,15 @@ static cudaError_t launch_route_kernel(const LaunchCtx &c, const float *logits) 
   return launch_kernel(route_kernel<8>, grid, block, 0, c.stream, a);
 }
 
-static bool tree_router_takes(const LaunchCtx &c) { return c.M <= kMaxTokChunk && c.desc->n_experts <= kTreeMaxN; }
+static bool tree_router_mma(const LaunchCtx &c) { return is_16bit(c.desc->dtype) && c.desc->d % (32 * kTreeWarps) == 0; }
+
+// On the tensor cores up to the 768 tokens from which the 64 x 16 router takes over (a layer of 64 experts, router_mma_kernel
+// / this one: 129 tokens 92.4 / 90.3 us, 255 108.0 / 105.7, 400 127.1 / 123.8, 767 244.0 / 242.1; 128 experts, 500 tokens
+// 201.7 / 197.3).  On the CUDA cores a CTA takes two tokens only and reads its 16 router rows again for every pair: 128
+// tokens, beyond which router_topk_kernel's eight are better (fp32, 200 tokens 698 / 704 us, 600 1912 / 1943).
+static bool tree_router_takes(const LaunchCtx &c) {
+  return c.desc->n_experts <= kTreeMaxN && c.M <= (tree_router_mma(c) ? 767 : kMaxTokChunk);
+}
 
 template <typename T, bool kMma>
 static cudaError_t launch_tree_router_t(const LaunchCtx &c, const void *hidden) {
@@ -1416,7 +1424,7 @@ static cudaError_t launch_tree_router_t(const LaunchCtx &c, const void *hidden) 
 template <typename T>
 static cudaError_t launch_tree_router(const LaunchCtx &c, const void *hidden) {
   if constexpr (sizeof(T) == 2)
-    if (c.desc->d % (32 * kTreeWarps) == 0) return launch_tree_router_t<T, true>(c, hidden);
+    if (tree_router_mma(c)) return launch_tree_router_t<T, true>(c, hidden);
   return launch_tree_router_t<T, false>(c, hidden);
 }
 
