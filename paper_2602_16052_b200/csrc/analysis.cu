@@ -39,11 +39,12 @@ __device__ __forceinline__ double warp_sum(double v) {
 // products instead of eight, and the rows come from L1 after the first read.  Twelve warps are one round of k = 8.
 constexpr int kGramThreads = 384, kGramB = 4;
 
-__global__ void __launch_bounds__(kGramThreads) gram_kernel(const float *__restrict__ y, const float *__restrict__ gate_w,
-                                                            const int *__restrict__ tokslot2row,
+__global__ void __launch_bounds__(kGramThreads) gram_kernel(const float *y, const float *gate_w, const int *tokslot2row,
                                                             double *__restrict__ gram, int *__restrict__ row2slot,
                                                             int d, int k) {
   const int t = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  pdl_trigger();
+  pdl_wait();
   if (threadIdx.x < k) {
     const int row = tokslot2row[(size_t)t * k + threadIdx.x];
     if (row >= 0) row2slot[row] = threadIdx.x;
@@ -95,7 +96,7 @@ __global__ void __launch_bounds__(kGramThreads) gram_kernel(const float *__restr
   }
 }
 
-// Greedy loop of Eq. 6 in one CTA.  gain(row) = 2 * sum of the row's Gram entries over the token's experts outside S,
+// Greedy loop of Eq. 6 in one CTA, for trees that greedy_rows_kernel below does not take.  gain(row) = 2 * sum of the row's Gram entries over the token's experts outside S,
 // minus its own: kept per routed row, so that a step recomputes only the rows of tokens that hold the expert just
 // picked (the same sum in the same order as from scratch) and otherwise adds up kept numbers.  Eight lanes take one
 // expert: they stride its rows in gather order and their partial sums meet in a shuffle tree, the same shape for every
@@ -140,8 +141,8 @@ constexpr size_t kGreedySmem = 200 * 1024;
 
 // gain_mem: scratch, one double per routed row; used when the working set stays in global memory (in_smem = 0).
 __global__ void __launch_bounds__(kGreedyThreads) greedy_kernel(
-    const double *gram, const int *assign_idx, const int *__restrict__ offset, const int *perm_row2tok,
-    const int *tokslot2row, const int *__restrict__ row2slot, const int *__restrict__ status, double *gain_mem, int M,
+    const double *gram, const int *assign_idx, const int *offset, const int *perm_row2tok,
+    const int *tokslot2row, const int *row2slot, const int *status, double *gain_mem, int M,
     int N, int k, int n_pick, int in_smem, RankingResult res) {
   extern __shared__ double s_work[];
   __shared__ unsigned char s_in[kMaxExperts];
@@ -150,6 +151,7 @@ __global__ void __launch_bounds__(kGreedyThreads) greedy_kernel(
   __shared__ int s_offset[kMaxExperts + 1];
   __shared__ double s_part[kGreedyThreads / 32];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  pdl_wait();
   for (int i = tid; i < N; i += kGreedyThreads) s_in[i] = 0;
   for (int i = tid; i <= N; i += kGreedyThreads) s_offset[i] = offset[i];
   double *gain = gain_mem;
@@ -240,6 +242,138 @@ __global__ void __launch_bounds__(kGreedyThreads) greedy_kernel(
   }
 }
 
+// The same loop for trees whose routed rows fit the registers of one CTA: up to 512 * ROWS (token, slot) pairs of k <= 8.
+// A thread keeps its pairs' Gram rows, the experts of their tokens and which of those are still outside S, so a pick is
+// answered by a compare and at most eight additions without a load, and a step is two barriers with an expert sum and an
+// argmax between them.  The sums are those of greedy_kernel in its order (the energy of the empty set apart, which is
+// added up pair by pair).  What bounds that one was a step's chain of dependent shared-memory loads (picked expert ->
+// its rows -> their tokens -> slots -> membership), integer divisions and a third barrier.  us a ranking of the first 32 of
+// 64 experts, layer pass included: 63 tokens 228 -> 188, 127 265 -> 213, 15 tokens (16 picks) 151 -> 134 (with the Gram
+// kernel and this one launched behind the layer's CTAs instead of behind its end).  A step is 0.9 us: sums 0.35, argmax
+// 0.1, the pick's rows 0.25, barriers.
+template <int ROWS, int W>
+__global__ void __launch_bounds__(kGreedyThreads) greedy_rows_kernel(
+    const double *gram, const int *assign_idx, const int *offset, const int *tokslot2row, const int *status, int M, int N,
+    int k, int n_pick, RankingResult res) {
+  __shared__ double s_row[kGreedyThreads * ROWS];         // gains of the routed rows, in gather order
+  __shared__ double s_gain[kMaxExperts];
+  __shared__ unsigned long long s_key[kMaxExperts];
+  __shared__ int s_offset[kMaxExperts + 1];
+  __shared__ double s_part[kGreedyThreads / 32];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  pdl_wait();
+  for (int i = tid; i <= N; i += kGreedyThreads) s_offset[i] = offset[i];
+  double G[ROWS][8], own[ROWS];
+  unsigned id[ROWS][2], out[ROWS][2];      // experts of the token's slots, a byte each; 0xff where outside S, else 0
+  int row[ROWS];
+  double acc = 0.0;
+#pragma unroll
+  for (int q = 0; q < ROWS; ++q) {
+    // (no load behind a branch: they would be waited for one by one)
+    const int pair = tid + q * kGreedyThreads, p = min(pair, M * k - 1), t = p / k, a = p - t * k;
+    int e[8];
+#pragma unroll
+    for (int b = 0; b < 8; ++b) {
+      e[b] = assign_idx[t * k + min(b, k - 1)];
+      G[q][b] = gram[(size_t)p * k + min(b, k - 1)];
+    }
+    row[q] = tokslot2row[p];
+    own[q] = gram[(size_t)p * k + a];
+    if (pair >= M * k) row[q] = -1;
+    id[q][0] = id[q][1] = out[q][0] = out[q][1] = 0u;
+#pragma unroll
+    for (int b = 0; b < 8; ++b) {
+      if (pair >= M * k || b >= k) G[q][b] = 0.0;
+      if (b < k && e[b] >= 0) {
+        id[q][b >> 2] |= (unsigned)e[b] << (8 * (b & 3));
+        out[q][b >> 2] |= 0xffu << (8 * (b & 3));
+      }
+      acc += G[q][b];
+    }
+  }
+  // objective of the empty set: sum_t || O*_t ||^2 = sum_t sum_{a,b} G_t[a][b], in a fixed order
+  double err = 0.0;
+  acc = warp_sum(acc);
+  if (lane == 0) s_part[warp] = acc;
+  __syncthreads();
+  for (int w = 0; w < kGreedyThreads / 32; ++w) err += s_part[w];
+  if (tid == 0) {
+    *res.gold = err;
+    *res.status = *status;
+  }
+  auto store_gain = [&](int q) {
+    double cross = 0.0;
+#pragma unroll
+    for (int b = 0; b < 8; ++b)
+      if ((out[q][b >> 2] >> (8 * (b & 3))) & 1u) cross += G[q][b];
+    if (row[q] >= 0) s_row[row[q]] = 2.0 * cross - own[q];
+  };
+#pragma unroll
+  for (int q = 0; q < ROWS; ++q) store_gain(q);
+  __syncthreads();
+  unsigned taken = 0;        // this lane's experts lane, lane + 32, ... that are in S, or beyond the last: bit i / 32
+#pragma unroll
+  for (int slot = 0; slot < W; ++slot)
+    if (lane + 32 * slot >= N) taken |= 1u << slot;
+  for (int step = 0; step < n_pick; ++step) {
+    // eight lanes an expert
+    for (int i0 = 0; i0 < N; i0 += kGreedyThreads / 8) {
+      const int i = i0 + (tid >> 3), sub = tid & 7;
+      double g = 0.0;
+      if (i < N) {
+        const int end = s_offset[i + 1];
+#pragma unroll 4
+        for (int r = s_offset[i] + sub; r < end; r += 8) g += s_row[r];
+      }
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1) {
+        int lo = __double2loint(g), hi = __double2hiint(g);
+        lo = __shfl_xor_sync(kFullMask, lo, o);
+        hi = __shfl_xor_sync(kFullMask, hi, o);
+        g += __hiloint2double(hi, lo);
+      }
+      if (sub == 0 && i < N) {
+        s_gain[i] = g;
+        s_key[i] = order_bits(g);
+      }
+    }
+    __syncthreads();
+    // every warp finds the largest gain for itself (ties: lower index)
+    unsigned long long best = 0;
+    unsigned best_slot = 32;        // none
+#pragma unroll
+    for (int slot = W - 1; slot >= 0; --slot) {      // descending: an equal gain goes to the lower index
+      const unsigned long long key = s_key[lane + 32 * slot];
+      if (!((taken >> slot) & 1u) && key >= best) {
+        best = key;
+        best_slot = slot;
+      }
+    }
+    const unsigned hi = __reduce_max_sync(kFullMask, (unsigned)(best >> 32));
+    const unsigned lo = __reduce_max_sync(kFullMask, (unsigned)(best >> 32) == hi ? (unsigned)best : 0u);
+    const bool mine = best_slot < 32 && (unsigned)(best >> 32) == hi && (unsigned)best == lo;
+    const int best_i = (int)__reduce_min_sync(kFullMask, mine ? best_slot * 32 + lane : 0x7fffffffu);
+    if (lane == (best_i & 31)) taken |= 1u << (best_i >> 5);
+    err -= s_gain[best_i];
+    if (tid == 0) {
+      res.order[step] = best_i;
+      res.objective[step] = err;
+    }
+    // rows of the tokens that hold it
+    const unsigned pattern = (unsigned)best_i * 0x01010101u;
+#pragma unroll
+    for (int q = 0; q < ROWS; ++q) {
+      const unsigned hit0 = __vcmpeq4(id[q][0], pattern) & out[q][0], hit1 = __vcmpeq4(id[q][1], pattern) & out[q][1];
+      if (hit0 | hit1) {
+        out[q][0] &= ~hit0;
+        out[q][1] &= ~hit1;
+        store_gain(q);
+      }
+    }
+    __syncthreads();
+  }
+}
+
 // sum (a - b)^2 and sum b^2 over n elements: every CTA reduces one contiguous slice in a fixed order,
 // the partial sums are added by a one-CTA launch.
 template <typename T>
@@ -287,20 +421,32 @@ __global__ void sqdiff_final_kernel(const double *__restrict__ partial, int n_pa
 }  // namespace
 
 cudaError_t launch_gram(const LaunchCtx &c, double *gram, int *row2slot) {
-  gram_kernel<<<c.M, kGramThreads, 0, c.stream>>>(c.ws->y, c.ws->gate_w, c.ws->tokslot2row, gram, row2slot, c.desc->d, c.k);
-  return cudaGetLastError();
+  return launch_kernel(gram_kernel, dim3(c.M), dim3(kGramThreads), 0, c.stream, (const float *)c.ws->y,
+                       (const float *)c.ws->gate_w, (const int *)c.ws->tokslot2row, gram, row2slot, c.desc->d, c.k);
 }
 
 cudaError_t launch_greedy(const LaunchCtx &c, const double *gram, const int *row2slot, int n_pick, double *row_gain,
                           const RankingResult &res) {
+  const int pairs = c.M * c.k;
+  if (c.k <= 8 && pairs <= 4 * kGreedyThreads) {
+    auto go = [&](auto kernel) {
+      return launch_kernel(kernel, dim3(1), dim3(kGreedyThreads), 0, c.stream, gram, (const int *)c.ws->assign_idx,
+                           (const int *)c.ws->offset, (const int *)c.ws->tokslot2row, (const int *)c.ws->status, c.M,
+                           c.desc->n_experts, c.k, n_pick, res);
+    };
+    const bool narrow = c.desc->n_experts <= 64;
+    if (pairs <= kGreedyThreads) return narrow ? go(greedy_rows_kernel<1, 2>) : go(greedy_rows_kernel<1, 8>);
+    if (pairs <= 2 * kGreedyThreads) return narrow ? go(greedy_rows_kernel<2, 2>) : go(greedy_rows_kernel<2, 8>);
+    return narrow ? go(greedy_rows_kernel<4, 2>) : go(greedy_rows_kernel<4, 8>);
+  }
   const size_t bytes = greedy_bytes(c.M, c.k);
   const bool in_smem = bytes <= kGreedySmem;
   cudaError_t e = cudaFuncSetAttribute(greedy_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGreedySmem);
   if (e != cudaSuccess) return e;
-  greedy_kernel<<<1, kGreedyThreads, in_smem ? bytes : 0, c.stream>>>(
-      gram, c.ws->assign_idx, c.ws->offset, c.ws->perm_row2tok, c.ws->tokslot2row, row2slot, c.ws->status, row_gain, c.M,
-      c.desc->n_experts, c.k, n_pick, in_smem, res);
-  return cudaGetLastError();
+  return launch_kernel(greedy_kernel, dim3(1), dim3(kGreedyThreads), in_smem ? bytes : 0, c.stream, gram,
+                       (const int *)c.ws->assign_idx, (const int *)c.ws->offset, (const int *)c.ws->perm_row2tok,
+                       (const int *)c.ws->tokslot2row, row2slot, (const int *)c.ws->status, row_gain, c.M,
+                       c.desc->n_experts, c.k, n_pick, (int)in_smem, res);
 }
 
 cudaError_t launch_sqdiff(const void *a, const void *b, size_t n, int dtype, double *partial, double *out,

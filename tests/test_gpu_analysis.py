@@ -206,6 +206,31 @@ def test_ranking_with_the_working_set_in_global_memory():
         layer.destroy()
 
 
+@pytest.mark.parametrize("M,k,N", [(1, 1, 3), (5, 3, 130), (64, 8, 64), (65, 8, 100), (128, 8, 64), (129, 8, 65), (256, 8, 64),
+                                   (257, 8, 64), (40, 9, 64)])
+def test_greedy_loop_at_the_edges_of_its_row_counts(M, k, N):
+    """One, two and four pairs per thread, full and one over, fewer than eight slots, more than 64 experts, and the sizes
+    beyond that the general kernel takes.  The loop is replayed in fp64 on the GPU's own Gram matrices: every pick has the
+    largest gain up to the rounding of a sum of M * k terms (1e-12 of the gold energy)."""
+    cfg = synth.CONFIGS["olmoe"].with_(d=128, f=128, n_experts=N, k=k)
+    case = H.make_case(cfg, M, seed=M)
+    layer = make_layer(case, M, k, out_dtype=torch.float32)
+    n_pick = min(N, 40)
+    order, obj, gold = layer.oracle_ranking(case["hidden"], k, n_pick)
+    G, idx = np.asarray(layer.get_gram()), layer.get_routing()["assign_idx"]
+    assert gold == pytest.approx(G.sum(), rel=1e-12)
+    left, err = np.ones((M, k)), G.sum()
+    for pick, o in zip(order, obj):
+        gain = 2.0 * (G * left[:, None, :]).sum(2) - np.diagonal(G, axis1=1, axis2=2)
+        total = np.bincount(idx.ravel(), weights=(gain * left).ravel(), minlength=N)
+        total[order[:list(order).index(pick)]] = -np.inf
+        assert total[pick] >= total.max() - 1e-12 * gold
+        err -= total[pick]
+        assert o == pytest.approx(err, rel=0, abs=1e-12 * gold)
+        left[idx == pick] = 0.0
+    layer.destroy()
+
+
 def test_analysis_argument_errors():
     m = ms()
     cfg = synth.CONFIGS["olmoe"].with_(f=128, n_experts=16)
