@@ -652,7 +652,6 @@ struct RouteArgs {
 };
 
 constexpr int kRouteWarps = 8;      // tokens per CTA of route_kernel
-constexpr int kMaxRouteWarps = 16;         // ... of any kernel that uses RouteShared
 constexpr int kColmaskCache = 1024; // words of the expert x token bit matrix the last CTA keeps in shared memory
 
 // Probability of expert `idx` from the row a warp holds in registers (lane l owns experts l, l+32, ...).
@@ -670,11 +669,9 @@ __device__ __forceinline__ double row_value(const double (&p)[W], int idx) {
 
 // Re-routing of one token (Eq. 7 / Eq. 8) with its mixing weights (Section 3.3); lane r owns slot r.
 // key[] / p[] are the token's logit keys and probabilities, valid says which slots exist.
-// The kept experts are recorded in the call's accumulators, or (kOneCta) in the CTA's own bit matrix, one word per expert.
-template <int W, bool kOneCta = false>
+template <int W>
 __device__ __forceinline__ void token_reroute(const RouteArgs &a, int t, int nS, const uint32_t *s_Smask,
-                                              const uint32_t (&key)[W], const double (&p)[W], int nat, int lane,
-                                              unsigned *s_colmask = nullptr, short *s_assign = nullptr) {
+                                              const uint32_t (&key)[W], const double (&p)[W], int nat, int lane) {
   const Workspace &ws = a.ws;
   const int k = a.k;
   const bool nat_kept = nat >= 0 && ((s_Smask[nat >> 5] >> (nat & 31)) & 1u);
@@ -720,27 +717,20 @@ __device__ __forceinline__ void token_reroute(const RouteArgs &a, int t, int nS,
   if (lane < k) {
     ws.assign_idx[(size_t)t * k + lane] = mine;
     ws.gate_w[(size_t)t * k + lane] = mine >= 0 ? (float)(p_mine / denom) : 0.f;
-    if constexpr (kOneCta) {
-      s_assign[t * k + lane] = (short)mine;
-      if (mine >= 0) atomicOr(s_colmask + mine, 1u << t);
-    } else if (mine >= 0) {
+    if (mine >= 0) {
       atomicAdd(ws.count_acc + mine, 1);
       atomicOr(ws.colmask + (size_t)mine * ((a.M + 31) >> 5) + (t >> 5), 1u << (t & 31));
     }
   }
 }
 
-// Shared memory of the shortlist, for up to NMAX experts, ...
-template <int NMAX>
-struct ShortlistShared {
-  unsigned long long score[NMAX];     // ranking key (score + 1, or 0 for a non-candidate)
-  int cand[NMAX];
-  int Srank[NMAX];
+// Shared memory of route_kernel.  It stays below 16 KB, so that a CTA of the FFN kernel fits beside it.
+struct RouteShared {
+  unsigned long long score[kMaxExperts];     // ranking key (score + 1, or 0 for a non-candidate)
+  int cand[kMaxExperts];
+  int Srank[kMaxExperts];
   uint32_t Smask[kMaskWords];
-  unsigned long long warp_tot[kMaxRouteWarps];
-};
-// ... and of route_kernel, which stays below 16 KB, so that a CTA of the FFN kernel fits beside it.
-struct RouteShared : ShortlistShared<kMaxExperts> {
+  unsigned long long warp_tot[kRouteWarps];
   unsigned long long fx[kMaxExperts];        // fixed-point score
   unsigned colmask[kColmaskCache];
   int count[kMaxExperts];
@@ -758,10 +748,9 @@ struct Shortlist {
 // Shortlist (Section 3.2) from the scores (Eq. 5) and the union (Eq. 3), which the caller's thread i < N has put into
 // sh.cand[i] and sh.score[i]; every thread of the CTA takes part.  write_rank, publish: this CTA also writes out the
 // shortlist, and publishes it to the FFN kernel.
-template <int NMAX>
-__device__ __forceinline__ Shortlist pick_shortlist(const RouteArgs &a, ShortlistShared<NMAX> &sh, int in_union,
-                                                    bool write_rank, bool publish) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n_warps = blockDim.x >> 5;
+__device__ __forceinline__ Shortlist pick_shortlist(const RouteArgs &a, RouteShared &sh, int in_union, bool write_rank,
+                                                    bool publish) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int N = a.N;
   const Workspace &ws = a.ws;
   if (tid < kMaskWords) sh.Smask[tid] = 0u;
@@ -820,7 +809,7 @@ __device__ __forceinline__ Shortlist pick_shortlist(const RouteArgs &a, Shortlis
     int pos = __popc(bal & ((1u << lane) - 1u));
     for (int w = 0; w < warp; ++w) pos += (int)sh.warp_tot[w];
     nS_l = 0;
-    for (int w = 0; w < n_warps; ++w) nS_l += (int)sh.warp_tot[w];
+    for (int w = 0; w < kRouteWarps; ++w) nS_l += (int)sh.warp_tot[w];
     if (res) sh.Srank[pos] = e_r;
     __syncthreads();
   }
@@ -835,12 +824,10 @@ __device__ __forceinline__ Shortlist pick_shortlist(const RouteArgs &a, Shortlis
   return Shortlist{nS, nS_l, n_union};
 }
 
-// What remains once every token's kept experts are known: offsets, rows, work units and statistics, by one CTA.  kOneCta:
-// the kept experts lie in this CTA's shared memory (sh.colmask, one word per expert, and s_assign), else in the call's
-// accumulators, which are cleared for the next call.
-template <bool kOneCta>
-__device__ __forceinline__ void finish_call(const RouteArgs &a, RouteShared &sh, const Shortlist &sl, const short *s_assign) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n_warps = blockDim.x >> 5;
+// What remains once every token's kept experts are known: offsets, rows, work units and statistics, by the CTA that arrives
+// last; it clears the call's accumulators for the next one.
+__device__ __forceinline__ void finish_call(const RouteArgs &a, RouteShared &sh, const Shortlist &sl) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int M = a.M, N = a.N, k = a.k;
   const int mw = (a.M + 31) >> 5;     // words per expert row of the bit matrix in this call
   const Workspace &ws = a.ws;
@@ -850,8 +837,8 @@ __device__ __forceinline__ void finish_call(const RouteArgs &a, RouteShared &sh,
   const int used_words = (M + 31) >> 5;
   const bool cm_cached = N * used_words <= kColmaskCache;
   {
-    const int c = tid >= N ? 0 : kOneCta ? __popc(sh.colmask[tid]) : __ldcg(ws.count_acc + tid);
-    if (!kOneCta && cm_cached)
+    const int c = tid < N ? __ldcg(ws.count_acc + tid) : 0;
+    if (cm_cached)
       for (int i = tid; i < N * used_words; i += blockDim.x) sh.colmask[i] = __ldcg(ws.colmask + i);
     // work units and the active count cover the resident experts only; rows and offsets cover all
     const bool resident = tid >= a.res_first && tid < a.res_first + a.res_count;
@@ -916,7 +903,7 @@ __device__ __forceinline__ void finish_call(const RouteArgs &a, RouteShared &sh,
     }
     if (tid == 0) {
       int tot = 0;
-      for (int w = 0; w < n_warps; ++w) tot += (int)sh.warp_tot[w];
+      for (int w = 0; w < kRouteWarps; ++w) tot += (int)sh.warp_tot[w];
       sh.nchunks = tot;
     }
     __syncthreads();
@@ -953,7 +940,7 @@ __device__ __forceinline__ void finish_call(const RouteArgs &a, RouteShared &sh,
   }
 
   // The rest is three independent jobs, each latency-bound, run side by side:
-  //   warps 0-3  row of every (token, slot)       warps 4-6 (8-15)  work-unit list       warp 7  coverage
+  //   warps 0-3  row of every (token, slot)       warps 4-6  work-unit list       warp 7  coverage
   const int n_chunks = sh.nchunks;
   double cov = 0.0;
   if (warp < 4 && !a.rows_later) {
@@ -994,11 +981,11 @@ __device__ __forceinline__ void finish_call(const RouteArgs &a, RouteShared &sh,
         ws.tokslot2row[(size_t)tt * k + slot] = row;
       }
     }
-  } else if (warp >= 4 && warp != 7) {
+  } else if (warp >= 4 && warp < 7) {
     // work units (expert, token chunk, 128-row slab): all gate/up units, then all down
     // units, each group ordered by (expert, chunk, slab); ready counters and the dispenser start at 0
     if (a.tiles_up > 0) {
-      const int lt = warp < 7 ? tid - 128 : tid - 160, nthr = blockDim.x - 160;
+      const int lt = tid - 128, nthr = 96;
       const int n_up = n_chunks * a.tiles_up, n_down = n_chunks * a.tiles_down;
       for (int i = lt; i < n_chunks; i += nthr) ws.ready[i] = 0;
       for (int u = lt; u < n_up + n_down; u += nthr) {
@@ -1056,9 +1043,8 @@ __device__ __forceinline__ void finish_call(const RouteArgs &a, RouteShared &sh,
     st.weight_bytes = (long long)sh.nactive * a.expert_bytes;
     *ws.stats = st;
     *ws.status = 0;
-    if (!kOneCta) *ws.arrive_route = 0;
+    *ws.arrive_route = 0;
   }
-  if (kOneCta) return;            // nothing of the call's accumulators was used
   __syncthreads();
   for (int i = tid; i < N; i += blockDim.x) {
     ws.score_fx[i] = 0ull;
@@ -1125,7 +1111,7 @@ __global__ void __launch_bounds__(kRouteWarps * 32) route_kernel(RouteArgs a) {
     sh.score[tid] = sh.cand[tid] ? fx + 1ull : 0ull;        // ranking key: candidates first, then by score
     sh.fx[tid] = fx;
   }
-  const Shortlist sl = pick_shortlist<kMaxExperts>(a, sh, in_union, blockIdx.x == 0, blockIdx.x == 0 && ws.early_flag && !a.from_router);
+  const Shortlist sl = pick_shortlist(a, sh, in_union, blockIdx.x == 0, blockIdx.x == 0 && ws.early_flag && !a.from_router);
 
   // ---- re-routing (Eq. 7 / Eq. 8) and mixing weights (Section 3.3) of this warp's token
   if (t < M) token_reroute<W>(a, t, sl.nS, sh.Smask, key, p, nat, lane);
@@ -1138,7 +1124,7 @@ __global__ void __launch_bounds__(kRouteWarps * 32) route_kernel(RouteArgs a) {
   }
   __syncthreads();
   if (!sh.last) return;
-  finish_call<false>(a, sh, sl, nullptr);
+  finish_call(a, sh, sl);
 }
 
 // Shortlist from the completed scores and union, by one CTA, for the FFN kernel's CTAs that wait for it: as
