@@ -378,7 +378,8 @@ __global__ void __maxnreg__(80) ffn_tc_kernel(const __grid_constant__ TcMapsCall
       if (lane == 0 && t_first < (int)gridDim.x) {
         const int r = r_first;
         int v = -1;                      // the expert of rank r, plus one
-        if (a.static_nS > 0) {           // a fixed shortlist needs no publication: stream from the first cycle
+        if (r >= a.M * a.k) {            // more ranks than routed rows: the list does not hold this one for its rank's sake
+        } else if (a.static_nS > 0) {    // a fixed shortlist needs no publication: stream from the first cycle
           if (r < a.static_nS) v = a.static_order[r] + 1;
         } else if (r < a.n_words) {
           const long long t0 = clock64();
