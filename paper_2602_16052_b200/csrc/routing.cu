@@ -600,25 +600,45 @@ cudaError_t launch_router_logits(const LaunchCtx &c, const void *hidden) {
   return launch_router_t<float>(c, hidden);
 }
 
-// Softmax and top-k from caller-supplied logits: one warp per token.
-__global__ void __launch_bounds__(128) softmax_topk_kernel(const float *logits, double *prob, int *topk_idx,
-                                                           unsigned long long *score_fx, int *natcnt, int *early_flag,
-                                                           unsigned *colmask, int M, int N, int k) {
-  const int t = blockIdx.x * 4 + (threadIdx.x >> 5);
+// Softmax and top-k of finished logits: one warp per token, sixteen per CTA, whose contributions to the scores and the
+// union are added up in shared memory first, so that an expert's counter takes one atomic per CTA and not per token (they
+// are performed one after the other).  us a layer, an atomic per token / this: 2048 tokens of 64 experts 368 / 360, 1000 of
+// 128 experts 273 / 266.
+constexpr int kSoftmaxWarps = 16;
+
+__global__ void __launch_bounds__(kSoftmaxWarps * 32) softmax_topk_kernel(const float *logits, double *prob, int *topk_idx,
+                                                                          unsigned long long *score_fx, int *natcnt,
+                                                                          int *early_flag, unsigned *colmask, int M, int N,
+                                                                          int k) {
+  extern __shared__ unsigned long long s_fx[];            // [kSoftmaxWarps][N], then the counts [N]
+  int *s_nat = reinterpret_cast<int *>(s_fx + kSoftmaxWarps * N);
+  const int warp = threadIdx.x >> 5, t = blockIdx.x * kSoftmaxWarps + warp;
+  for (int i = threadIdx.x; i < kSoftmaxWarps * N; i += blockDim.x) s_fx[i] = 0ull;
+  for (int i = threadIdx.x; i < N; i += blockDim.x) s_nat[i] = 0;
+  __syncthreads();
   pdl_trigger();
   pdl_wait();
   if (early_flag && blockIdx.x == 0)
     for (int i = threadIdx.x; i < N; i += blockDim.x) early_flag[i] = 0;
   clear_colmask(colmask, N * ((M + 31) >> 5));
   if (t < M)
-    token_phase(logits + (size_t)t * N, N, k, prob + (size_t)t * N, topk_idx + (size_t)t * k, score_fx, natcnt,
+    token_phase(logits + (size_t)t * N, N, k, prob + (size_t)t * N, topk_idx + (size_t)t * k, s_fx + warp * N, s_nat,
                 threadIdx.x & 31);
+  __syncthreads();
+  for (int i = threadIdx.x; i < N; i += blockDim.x) {
+    unsigned long long fx = 0ull;
+#pragma unroll
+    for (int w = 0; w < kSoftmaxWarps; ++w) fx += s_fx[w * N + i];
+    if (fx) atomicAdd(score_fx + i, fx);
+    if (s_nat[i]) atomicAdd(natcnt + i, s_nat[i]);
+  }
 }
 
 static cudaError_t launch_softmax_topk(const LaunchCtx &c, const float *logits, int *early_flag) {
-  return launch_kernel(softmax_topk_kernel, dim3((c.M + 3) / 4), dim3(128), 0, c.stream, logits, c.ws->prob,
-                       c.ws->topk_idx, c.ws->score_fx, c.ws->natcnt_acc, early_flag, c.ws->colmask, c.M,
-                       c.desc->n_experts, c.k);
+  const int N = c.desc->n_experts;
+  return launch_kernel(softmax_topk_kernel, dim3((c.M + kSoftmaxWarps - 1) / kSoftmaxWarps), dim3(kSoftmaxWarps * 32),
+                       (size_t)N * (kSoftmaxWarps * sizeof(unsigned long long) + sizeof(int)), c.stream, logits, c.ws->prob,
+                       c.ws->topk_idx, c.ws->score_fx, c.ws->natcnt_acc, early_flag, c.ws->colmask, c.M, N, c.k);
 }
 
 __device__ __forceinline__ double shfl_double(double x, int src) {
