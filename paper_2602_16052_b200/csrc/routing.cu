@@ -1318,26 +1318,30 @@ __global__ void __maxnreg__(136) tree_router_kernel(const T *__restrict__ hidden
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         const int jh = j0 + h * 32 * VEC * U;
+        // every load of both tokens before the first FMA and none behind a branch; what lies beyond d is not used
+        uint4 X[TOK][U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int off = jh + u * 32 * VEC < d ? jh + u * 32 * VEC : 0;
+#pragma unroll
+          for (int tt = 0; tt < TOK; ++tt)                      // clamp: a token beyond M repeats the last row
+            X[tt][u] = *reinterpret_cast<const uint4 *>(hidden + (size_t)min(t0 + tt, M - 1) * d + off);
+        }
         if (j0 != lane * VEC) {
 #pragma unroll
-          for (int u = 0; u < U; ++u)
-            if (jh + u * 32 * VEC < d) {
-              W0[h * U + u] = *reinterpret_cast<const uint4 *>(w0 + jh - lane * VEC + u * 32 * VEC);
-              W1[h * U + u] = *reinterpret_cast<const uint4 *>(w1 + jh - lane * VEC + u * 32 * VEC);
-            }
+          for (int u = 0; u < U; ++u) {
+            const int off = jh + u * 32 * VEC < d ? jh + u * 32 * VEC - lane * VEC : 0;
+            W0[h * U + u] = *reinterpret_cast<const uint4 *>(w0 + off);
+            W1[h * U + u] = *reinterpret_cast<const uint4 *>(w1 + off);
+          }
         }
 #pragma unroll
-        for (int tt = 0; tt < TOK; ++tt) {
-          const T *hr = hidden + (size_t)min(t0 + tt, M - 1) * d;      // clamp: a token beyond M repeats the last row
-          uint4 X[U];
+        for (int u = 0; u < U; ++u) {
+          if (jh + u * 32 * VEC < d) {
+            const T *ew0 = reinterpret_cast<const T *>(&W0[h * U + u]), *ew1 = reinterpret_cast<const T *>(&W1[h * U + u]);
 #pragma unroll
-          for (int u = 0; u < U; ++u)
-            if (jh + u * 32 * VEC < d) X[u] = *reinterpret_cast<const uint4 *>(hr + jh + u * 32 * VEC);
-#pragma unroll
-          for (int u = 0; u < U; ++u) {
-            if (jh + u * 32 * VEC < d) {
-              const T *ew0 = reinterpret_cast<const T *>(&W0[h * U + u]), *ew1 = reinterpret_cast<const T *>(&W1[h * U + u]);
-              const T *eh = reinterpret_cast<const T *>(&X[u]);
+            for (int tt = 0; tt < TOK; ++tt) {
+              const T *eh = reinterpret_cast<const T *>(&X[tt][u]);
 #pragma unroll
               for (int v = 0; v < VEC; ++v) {
                 acc[0][tt] = fmaf(to_float(ew0[v]), to_float(eh[v]), acc[0][tt]);
