@@ -1208,8 +1208,10 @@ __device__ __forceinline__ void publish_shortlist(const RouteArgs &a, unsigned l
 //     that kernel ends.
 //   * The FFN kernel is released by this kernel's CTAs (through route_kernel and the gather, which release at once) and
 //     is resident when the shortlist comes.  Its control words have been reset by then: by a cluster of its own, whose
-//     release follows a fence.
-//   * The last CTA to arrive publishes the shortlist; route_kernel finds it again from the same scores.
+//     release follows a fence.  That cluster is the first of the grid, because the FFN kernel is released by it too.
+//   * The last CTA to arrive publishes the shortlist; route_kernel finds it again from the same scores.  The CTA that
+//     resets the shortlist words counts among those that arrive: the grid need not be resident at once (136 registers are
+//     one CTA per SM, and other handles' kernels may hold SMs), so nothing else orders its zeros before the publication.
 // ---------------------------------------------------------------------------
 constexpr int kTreeWarps = 8, kTreeExperts = 16, kTreeMaxN = 128;
 template <bool kMma> constexpr int kTreeTokens = kMma ? 8 : 2;      // token tile of a cluster
@@ -1228,15 +1230,28 @@ __global__ void __maxnreg__(136) tree_router_kernel(const T *__restrict__ hidden
   const int M = a.M, N = a.N, k = a.k;
   const Workspace &ws = a.ws;
   const uint32_t C = gridDim.x;                       // CTAs of a cluster: the experts of one token tile
-  if (blockIdx.y == gridDim.y - 1) {                  // a cluster of its own prepares the FFN kernel's control words
+  // The CTA that arrives last publishes the shortlist: every token has added its scores by then, and the shortlist words
+  // have been reset (the resetting CTA arrives too, so its zeros cannot come after the publication).
+  auto arrive_and_publish = [&]() {
+    __syncthreads();
+    if (tid == 0) {
+      const int n = (int)(C * (gridDim.y - 1)) + 1;       // the CTAs of the token tiles and the one that resets
+      s_last = arrive_acq_rel(ws.arrive) == n - 1;
+      if (s_last) ws.arrive[0] = 0;
+    }
+    __syncthreads();
+    if (s_last) publish_shortlist(a, sh.score);
+  };
+  if (blockIdx.y == 0) {                              // a cluster of its own prepares the FFN kernel's control words
     pdl_wait();
     if (blockIdx.x == 0) reset_ffn_control(ws.early_flag, N, ws.unit_counter, 1);
     pdl_trigger();
     for (int i = (int)blockIdx.x * blockDim.x + tid; i < N * ((M + 31) >> 5); i += C * blockDim.x) ws.colmask[i] = 0u;
+    if (publish && blockIdx.x == 0) arrive_and_publish();
     return;
   }
   const uint32_t rank = blockIdx.x;
-  const int e0 = (int)rank * kTreeExperts, t0 = (int)blockIdx.y * TOK;
+  const int e0 = (int)rank * kTreeExperts, t0 = (int)(blockIdx.y - 1) * TOK;
   // C is a power of two
   const int c_bits = 31 - __clz(C), slots = (TOK + (int)C - 1) >> c_bits;      // tokens of this CTA
 
@@ -1370,16 +1385,7 @@ __global__ void __maxnreg__(136) tree_router_kernel(const T *__restrict__ hidden
       token_phase(s_z + q * N, N, k, ws.prob + (size_t)t * N, ws.topk_idx + (size_t)t * k, ws.score_fx, ws.natcnt_acc, lane,
                   1 + (item & 1));
   }
-  if (!publish) return;
-  // the CTA that arrives last knows every score: it publishes the shortlist
-  __syncthreads();
-  if (tid == 0) {
-    const int n = (int)(gridDim.x * (gridDim.y - 1));
-    s_last = arrive_acq_rel(ws.arrive) == n - 1;
-    if (s_last) ws.arrive[0] = 0;
-  }
-  __syncthreads();
-  if (s_last) publish_shortlist(a, sh.score);
+  if (publish) arrive_and_publish();
 }
 
 static RouteArgs route_args(const LaunchCtx &c, const float *logits) {
