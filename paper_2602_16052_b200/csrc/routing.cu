@@ -1199,10 +1199,8 @@ __device__ __forceinline__ void publish_shortlist(const RouteArgs &a, unsigned l
 // 72.5 -> 69.9).
 //   * A cluster of CTAs takes a token tile, each CTA 16 experts of it; the logits of a token meet in the shared memory
 //     of the CTA that owns the token (cluster_sync) instead of global memory and an arrival counter.
-//   * 16-bit layers: 16 experts x 8 tokens a CTA on mma.sync, K split over eight warps, every load of a batch issued
-//     before the first MMA and none behind a branch of its own (guarded loads were waited for one by one: 3300 cycles
-//     instead of 1100).  fp32 layers, and widths that do not split: 16 experts x 2 tokens on the CUDA cores, the sums of
-//     router_topk_kernel.
+//   * 16 experts x 8 tokens a CTA on mma.sync, K split over eight warps, every load of a batch issued before the first
+//     MMA and none behind a branch of its own (guarded loads were waited for one by one: 3300 cycles instead of 1100).
 //   * 8 warps of at most 136 registers and 5 KB of shared memory fit beside a CTA of the previous call's FFN kernel (10
 //     warps of 80), register file quarter by quarter, so that the CTAs are resident with their router rows loaded when
 //     that kernel ends.
@@ -1210,16 +1208,17 @@ __device__ __forceinline__ void publish_shortlist(const RouteArgs &a, unsigned l
 //     is resident when the shortlist comes.  Its control words have been reset by then: by a cluster of its own, whose
 //     release follows a fence.  That cluster is the first of the grid, because the FFN kernel is released by it too.
 //   * The last CTA to arrive publishes the shortlist; route_kernel finds it again from the same scores.  The CTA that
-//     resets the shortlist words counts among those that arrive: the grid need not be resident at once (136 registers are
-//     one CTA per SM, and other handles' kernels may hold SMs), so nothing else orders its zeros before the publication.
+//     resets the shortlist words counts among those that arrive: the grid need not be resident at once (beside a CTA of
+//     an FFN kernel an SM takes one, and clusters of eight leave SMs over), so nothing else orders its zeros before the
+//     publication.
 // ---------------------------------------------------------------------------
 constexpr int kTreeWarps = 8, kTreeExperts = 16, kTreeMaxN = 128;
-template <bool kMma> constexpr int kTreeTokens = kMma ? 8 : 2;      // token tile of a cluster
+constexpr int kTreeTokens = 8;                                      // token tile of a cluster
 
-template <typename T, bool kMma>
+template <typename T>
 __global__ void __maxnreg__(136) tree_router_kernel(const T *__restrict__ hidden, const T *__restrict__ Wr,
                                                     const float *__restrict__ bias, int d, int publish, RouteArgs a) {
-  constexpr int TOK = kTreeTokens<kMma>;
+  constexpr int TOK = kTreeTokens;
   __shared__ union {
     float part[kTreeWarps][kTreeExperts * TOK];      // partial dot products of the warps
     unsigned long long score[kTreeMaxN];
@@ -1255,26 +1254,23 @@ __global__ void __maxnreg__(136) tree_router_kernel(const T *__restrict__ hidden
   // C is a power of two
   const int c_bits = 31 - __clz(C), slots = (TOK + (int)C - 1) >> c_bits;      // tokens of this CTA
 
-  constexpr int VEC = 16 / sizeof(T), U = kMma ? 8 : 4;
-  const int g = lane >> 2, tg = lane & 3, kw = d / kTreeWarps;      // kMma: K range of this warp
-  // two router rows of this thread (kMma) or warp; a constant of the layer, so their start is fetched before the wait
-  const T *w0 = Wr + (kMma ? (size_t)min(e0 + g, N - 1) * d + warp * kw + tg * 8 : (size_t)min(e0 + warp, N - 1) * d + lane * VEC);
-  const T *w1 = Wr + (kMma ? (size_t)min(e0 + g + 8, N - 1) * d + warp * kw + tg * 8
-                           : (size_t)min(e0 + warp + kTreeWarps, N - 1) * d + lane * VEC);
-  // the bias of the logits this thread will finish (kMma: one; else lane 0 of a warp two)
-  auto bias_of = [&](int e) { return bias && e < N ? load_early(bias + e) : 0.f; };
-  const float b0 = bias_of(kMma ? e0 + tid / TOK % kTreeExperts : e0 + warp);
-  const float b1 = kMma ? 0.f : bias_of(e0 + warp + kTreeWarps);
-  uint4 W0[8], W1[8];
+  constexpr int U = 8;
+  const int g = lane >> 2, tg = lane & 3, kw = d / kTreeWarps;      // K range of this warp
+  // two router rows of this thread; a constant of the layer, so their start is fetched before the wait
+  const T *w0 = Wr + (size_t)min(e0 + g, N - 1) * d + warp * kw + tg * 8;
+  const T *w1 = Wr + (size_t)min(e0 + g + 8, N - 1) * d + warp * kw + tg * 8;
+  // the bias of the logit this thread will finish
+  const int e_bias = e0 + tid / TOK % kTreeExperts;
+  const float b0 = bias && e_bias < N ? load_early(bias + e_bias) : 0.f;
+  uint4 W0[U], W1[U];
 #pragma unroll
-  for (int s = 0; s < 8; ++s)
-    if (kMma || (lane + s * 32) * VEC < d) {
-      const int off = kMma ? (s * 32 < kw ? s * 32 : 0) : s * 32 * VEC;
-      W0[s] = load_early((const void *)(w0 + off));
-      W1[s] = load_early((const void *)(w1 + off));
-    }
+  for (int s = 0; s < U; ++s) {
+    const int off = s * 32 < kw ? s * 32 : 0;
+    W0[s] = load_early((const void *)(w0 + off));
+    W1[s] = load_early((const void *)(w1 + off));
+  }
   // ... and so are the kernel's arguments, whose lines of the constant bank each cost a miss at their first use
-  const T *hb = hidden + (kMma ? (size_t)min(t0 + g, M - 1) * d + warp * kw + tg * 8 : (size_t)0);
+  const T *hb = hidden + (size_t)min(t0 + g, M - 1) * d + warp * kw + tg * 8;
   asm volatile("" ::"l"(hb), "l"(ws.logits), "l"(ws.prob), "l"(ws.score_fx), "l"(ws.topk_idx), "l"(ws.natcnt_acc), "l"(ws.arrive),
                "l"(ws.early_flag), "r"(M), "r"(N), "r"(k), "r"(a.B), "r"(a.shortlist), "r"(a.res_first), "r"(publish));
   cluster_sync();        // the CTAs of the cluster have started
@@ -1286,96 +1282,45 @@ __global__ void __maxnreg__(136) tree_router_kernel(const T *__restrict__ hidden
     st_cluster(&s_z[(tl >> c_bits) * N + e], tl & (C - 1), __float_as_uint(z));
     ws.logits[(size_t)(t0 + tl) * N + e] = z;
   };
-  if constexpr (kMma) {
-    float c[4] = {0.f, 0.f, 0.f, 0.f};
-    // `steps` times 32 elements of K from k0 on; all loads are issued before the first MMA
-    auto block = [&](auto reload, int k0, int steps) {
-      uint4 X[U];
+  float c[4] = {0.f, 0.f, 0.f, 0.f};
+  // `steps` times 32 elements of K from k0 on; all loads are issued before the first MMA
+  auto block = [&](auto reload, int k0, int steps) {
+    uint4 X[U];
 #pragma unroll
-      for (int s = 0; s < U; ++s) {
-        const int off = k0 + (s < steps ? s : 0) * 32;        // (steps is U, or the remainder: those repeat the first)
-        X[s] = *reinterpret_cast<const uint4 *>(hb + off);
-        if constexpr (decltype(reload)::value) {
-          W0[s] = *reinterpret_cast<const uint4 *>(w0 + off);
-          W1[s] = *reinterpret_cast<const uint4 *>(w1 + off);
-        }
-      }
-      // Every MMA starts from zero and the running sums are kept in fp32 registers: a chain of MMAs on one accumulator
-      // rounds worse than the CUDA-core dot product.
-#pragma unroll
-      for (int s = 0; s < U; ++s) {
-        float lo[4] = {0.f, 0.f, 0.f, 0.f}, hi[4] = {0.f, 0.f, 0.f, 0.f};
-        mma_16816(lo, W0[s].x, W1[s].x, W0[s].y, W1[s].y, X[s].x, X[s].y, T());
-        mma_16816(hi, W0[s].z, W1[s].z, W0[s].w, W1[s].w, X[s].z, X[s].w, T());
-#pragma unroll
-        for (int q = 0; q < 4; ++q) c[q] += s < steps ? lo[q] + hi[q] : 0.f;
-      }
-    };
-    block(std::false_type(), 0, min(U, kw / 32));
-    for (int k0 = 32 * U; k0 < kw; k0 += 32 * U) block(std::true_type(), k0, min(U, (kw - k0) / 32));
-    float2 *part = reinterpret_cast<float2 *>(&sh.part[warp][g * TOK + 2 * tg]);
-    part[0] = make_float2(c[0], c[1]);
-    part[4 * TOK] = make_float2(c[2], c[3]);
-    __syncthreads();
-    if (tid < kTreeExperts * TOK) {
-      float v[kTreeWarps];
-#pragma unroll
-      for (int w = 0; w < kTreeWarps; ++w) v[w] = sh.part[w][tid];
-#pragma unroll
-      for (int o = 1; o < kTreeWarps; o <<= 1)
-#pragma unroll
-        for (int w = 0; w < kTreeWarps; w += 2 * o) v[w] += v[w + o];
-      finish_logit(tid % TOK, e0 + tid / TOK, v[0] + b0);
-    }
-  } else {
-    float acc[2][TOK] = {};
-    for (int j0 = lane * VEC; j0 < d; j0 += 64 * VEC * U) {
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int jh = j0 + h * 32 * VEC * U;
-        // every load of both tokens before the first FMA and none behind a branch; what lies beyond d is not used
-        uint4 X[TOK][U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const int off = jh + u * 32 * VEC < d ? jh + u * 32 * VEC : 0;
-#pragma unroll
-          for (int tt = 0; tt < TOK; ++tt)                      // clamp: a token beyond M repeats the last row
-            X[tt][u] = *reinterpret_cast<const uint4 *>(hidden + (size_t)min(t0 + tt, M - 1) * d + off);
-        }
-        if (j0 != lane * VEC) {
-#pragma unroll
-          for (int u = 0; u < U; ++u) {
-            const int off = jh + u * 32 * VEC < d ? jh + u * 32 * VEC - lane * VEC : 0;
-            W0[h * U + u] = *reinterpret_cast<const uint4 *>(w0 + off);
-            W1[h * U + u] = *reinterpret_cast<const uint4 *>(w1 + off);
-          }
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          if (jh + u * 32 * VEC < d) {
-            const T *ew0 = reinterpret_cast<const T *>(&W0[h * U + u]), *ew1 = reinterpret_cast<const T *>(&W1[h * U + u]);
-#pragma unroll
-            for (int tt = 0; tt < TOK; ++tt) {
-              const T *eh = reinterpret_cast<const T *>(&X[tt][u]);
-#pragma unroll
-              for (int v = 0; v < VEC; ++v) {
-                acc[0][tt] = fmaf(to_float(ew0[v]), to_float(eh[v]), acc[0][tt]);
-                acc[1][tt] = fmaf(to_float(ew1[v]), to_float(eh[v]), acc[1][tt]);
-              }
-            }
-          }
-        }
+    for (int s = 0; s < U; ++s) {
+      const int off = k0 + (s < steps ? s : 0) * 32;        // (steps is U, or the remainder: those repeat the first)
+      X[s] = *reinterpret_cast<const uint4 *>(hb + off);
+      if constexpr (decltype(reload)::value) {
+        W0[s] = *reinterpret_cast<const uint4 *>(w0 + off);
+        W1[s] = *reinterpret_cast<const uint4 *>(w1 + off);
       }
     }
+    // Every MMA starts from zero and the running sums are kept in fp32 registers: a chain of MMAs on one accumulator
+    // rounds worse than the CUDA-core dot product.
 #pragma unroll
-    for (int h = 0; h < 2; ++h)
+    for (int s = 0; s < U; ++s) {
+      float lo[4] = {0.f, 0.f, 0.f, 0.f}, hi[4] = {0.f, 0.f, 0.f, 0.f};
+      mma_16816(lo, W0[s].x, W1[s].x, W0[s].y, W1[s].y, X[s].x, X[s].y, T());
+      mma_16816(hi, W0[s].z, W1[s].z, W0[s].w, W1[s].w, X[s].z, X[s].w, T());
 #pragma unroll
-      for (int tt = 0; tt < TOK; ++tt) {
-        float z = acc[h][tt];
+      for (int q = 0; q < 4; ++q) c[q] += s < steps ? lo[q] + hi[q] : 0.f;
+    }
+  };
+  block(std::false_type(), 0, min(U, kw / 32));
+  for (int k0 = 32 * U; k0 < kw; k0 += 32 * U) block(std::true_type(), k0, min(U, (kw - k0) / 32));
+  float2 *part = reinterpret_cast<float2 *>(&sh.part[warp][g * TOK + 2 * tg]);
+  part[0] = make_float2(c[0], c[1]);
+  part[4 * TOK] = make_float2(c[2], c[3]);
+  __syncthreads();
+  if (tid < kTreeExperts * TOK) {
+    float v[kTreeWarps];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(kFull, z, o);
-        if (lane == 0) finish_logit(tt, e0 + warp + h * kTreeWarps, z + (h ? b1 : b0));
-      }
+    for (int w = 0; w < kTreeWarps; ++w) v[w] = sh.part[w][tid];
+#pragma unroll
+    for (int o = 1; o < kTreeWarps; o <<= 1)
+#pragma unroll
+      for (int w = 0; w < kTreeWarps; w += 2 * o) v[w] += v[w + o];
+    finish_logit(tid % TOK, e0 + tid / TOK, v[0] + b0);
   }
   cluster_sync();              // slot q of this CTA is token t0 + q * C + rank
   // softmax (Eq. 1), scores (Eq. 5), natural top-k (Eq. 2) and union (Eq. 3): two warps per token
@@ -1419,38 +1364,32 @@ static cudaError_t launch_route_kernel(const LaunchCtx &c, const float *logits) 
   return launch_kernel(route_kernel<8>, grid, block, 0, c.stream, a);
 }
 
-static bool tree_router_mma(const LaunchCtx &c) { return is_16bit(c.desc->dtype) && c.desc->d % (32 * kTreeWarps) == 0; }
-
-// On the tensor cores up to the 768 tokens from which the 64 x 16 router takes over (a layer of 64 experts, router_mma_kernel
+// Layers whose products run on the tensor cores (K splits over the eight warps into whole 32-element steps).  The others
+// stay with router_topk_kernel: a CUDA-core form of this kernel (16 experts x 2 tokens a CTA) read the router rows again for
+// every pair of tokens and was slower nearly everywhere.  us a call, router_topk_kernel / that form: fp32 15 tokens of d =
+// 256 25.4 / 25.8, d = 2048 63 tokens of 128 experts 284 / 292, 127 tokens 448 / 465; bf16 d = 384 1 token of 128 experts
+// 28.1 / 31.1, 32 tokens 38.6 / 44.8, 127 tokens 50.7 / 61.0; d = 1408 63 tokens of 64 experts 73.0 / 75.2; d = 1920 127
+// tokens of 128 experts 110 / 122; faster in one of 50 (d = 2944, 127 tokens of 32 experts 75.3 / 72.2).
+// Up to the 768 tokens from which the 64 x 16 router takes over (a layer of 64 experts, router_mma_kernel
 // / this one: 129 tokens 92.4 / 90.3 us, 255 108.0 / 105.7, 400 127.1 / 123.8, 767 244.0 / 242.1; 128 experts, 500 tokens
-// 201.7 / 197.3).  On the CUDA cores a CTA takes two tokens only and reads its 16 router rows again for every pair: 128
-// tokens, beyond which router_topk_kernel's eight are better (fp32, 200 tokens 698 / 704 us, 600 1912 / 1943).
+// 201.7 / 197.3).
 static bool tree_router_takes(const LaunchCtx &c) {
-  return c.desc->n_experts <= kTreeMaxN && c.M <= (tree_router_mma(c) ? 767 : kMaxTokChunk);
-}
-
-template <typename T, bool kMma>
-static cudaError_t launch_tree_router_t(const LaunchCtx &c, const void *hidden) {
-  const moespec_layer_desc &D = *c.desc;
-  RouteArgs a = route_args(c, c.ws->logits);
-  int C = 1;
-  while (C * kTreeExperts < D.n_experts) C *= 2;
-  const int tiles = (c.M + kTreeTokens<kMma> - 1) / kTreeTokens<kMma>;
-  return launch_kernel_cluster(tree_router_kernel<T, kMma>, dim3(C, tiles + 1), dim3(kTreeWarps * 32), C, c.stream,
-                               (const T *)hidden, (const T *)D.router_w, D.router_bias, D.d, a.from_router, a);
+  return is_16bit(c.desc->dtype) && c.desc->d % (32 * kTreeWarps) == 0 && c.desc->n_experts <= kTreeMaxN && c.M <= 767;
 }
 
 template <typename T>
 static cudaError_t launch_tree_router(const LaunchCtx &c, const void *hidden) {
-  if constexpr (sizeof(T) == 2)
-    if (tree_router_mma(c)) return launch_tree_router_t<T, true>(c, hidden);
-  return launch_tree_router_t<T, false>(c, hidden);
+  const moespec_layer_desc &D = *c.desc;
+  RouteArgs a = route_args(c, c.ws->logits);
+  int C = 1;
+  while (C * kTreeExperts < D.n_experts) C *= 2;
+  const int tiles = (c.M + kTreeTokens - 1) / kTreeTokens;
+  return launch_kernel_cluster(tree_router_kernel<T>, dim3(C, tiles + 1), dim3(kTreeWarps * 32), C, c.stream,
+                               (const T *)hidden, (const T *)D.router_w, D.router_bias, D.d, a.from_router, a);
 }
 
 static cudaError_t launch_router_for_tree(const LaunchCtx &c, const void *hidden) {
-  if (c.desc->dtype == MOESPEC_BF16) return launch_tree_router<__nv_bfloat16>(c, hidden);
-  if (c.desc->dtype == MOESPEC_FP16) return launch_tree_router<__half>(c, hidden);
-  return launch_tree_router<float>(c, hidden);
+  return c.desc->dtype == MOESPEC_BF16 ? launch_tree_router<__nv_bfloat16>(c, hidden) : launch_tree_router<__half>(c, hidden);
 }
 
 // Eq. 4: add the natural top-k counts of the last router launch to the calibration counters and
@@ -1605,11 +1544,8 @@ cudaError_t routing_configure() {
   set((const void *)route_kernel<2>);
   set((const void *)route_kernel<4>);
   set((const void *)route_kernel<8>);
-  set((const void *)tree_router_kernel<__nv_bfloat16, true>);
-  set((const void *)tree_router_kernel<__half, true>);
-  set((const void *)tree_router_kernel<__nv_bfloat16, false>);
-  set((const void *)tree_router_kernel<__half, false>);
-  set((const void *)tree_router_kernel<float, false>);
+  set((const void *)tree_router_kernel<__nv_bfloat16>);
+  set((const void *)tree_router_kernel<__half>);
   set((const void *)gather_rows_kernel);
   set((const void *)rows_gather_kernel);
   return e;
