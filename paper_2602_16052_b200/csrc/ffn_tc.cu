@@ -346,7 +346,8 @@ __global__ void __maxnreg__(80) ffn_tc_kernel(const __grid_constant__ TcMapsCall
     // each), because a single thread issuing 8-16 copies per stage would cap the SM's streaming rate.
     // Every unit, the first included, is a ticket from the dispenser.  The next unit is drawn a few
     // stages before the current one ends: early enough that the atomic and the descriptor load are
-    // hidden behind the stages still in flight, late enough that no CTA sits on units others could run.
+    // hidden behind the stages still in flight, late enough that no CTA sits on units others could run
+    // (nor while it waits for the rows of a down unit, below).
     int n_total = 0;                 // valid once `waited`
     bool waited = !a.early;          // has this warp waited for the routing kernels?
     uint32_t it = 0, qi = 0;
@@ -457,17 +458,18 @@ __global__ void __maxnreg__(80) ffn_tc_kernel(const __grid_constant__ TcMapsCall
       // A stage is armed and its weight copies issued by head(); its token-row copies by rows().  A down
       // unit reads h_mid, which is complete only when every gate/up slab of its expert has been published.
       int armed = 0;                                // stages of this unit whose barrier has been armed
+      int draw_kc = draw_at;                        // K iteration at which the next unit is drawn
       auto head = [&](int kc) {
         const uint32_t s = (it + kc) % n_stages, ph = ((it + kc) / n_stages) & 1u;
         const uint32_t full = bar_full + 8 * s;
         const uint32_t stage = smem_base + s * (uint32_t)a.stage_bytes;
-        if (kc == draw_at && !waited) {        // the unit list and the gathered rows are needed from here on
+        if (kc == draw_kc && !waited) {        // the unit list and the gathered rows are needed from here on
           pdl_wait();
           waited = true;
           n_total = a.n_units[0] + a.n_units[1];
         }
         if (lane == 0) {
-          if (kc == draw_at) u_next = atomicAdd(a.unit_counter, 1);
+          if (kc == draw_kc) u_next = atomicAdd(a.unit_counter, 1);
           if (!mbar_wait(bar_empty + 8 * s, ph ^ 1u, abort_flag, a.spin_limit)) ok = 0;
           else mbar_expect_tx(full, tx);
         }
@@ -514,6 +516,11 @@ __global__ void __maxnreg__(80) ffn_tc_kernel(const __grid_constant__ TcMapsCall
           // not yet: the weights of the first stages are requested BEFORE the wait, so that a CTA that runs
           // into the dependency keeps streaming instead of idling
           n_pre = k_iters < n_stages ? k_iters : n_stages;
+          // The next unit is drawn behind the wait: a CTA that stands here with two units leaves the second to run after
+          // the first, while CTAs that finish their gate/up units find nothing left to do.  (One token and 4 experts of
+          // d = 2944, 64 gate/up and 92 down units on 148 CTAs: 44.1 -> 39.2 us, 41.2 before trees this small had their
+          // early units limited to the routed ranks; 6 tokens, k = 2, d = 2048: 44.3 -> 39.1; trees of 63: the same.)
+          if (draw_at > 0 && draw_at < n_pre) draw_kc = min(n_pre, k_iters - 1);
           for (int kc = 1; kc < n_pre && ok; ++kc) head(kc);
           if (ok && lane == 0) {
             const long long t0 = clock64();
