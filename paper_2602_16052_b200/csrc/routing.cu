@@ -1346,7 +1346,18 @@ static RouteArgs route_args(const LaunchCtx &c, const float *logits) {
   a.rows_later = rows_in_row_kernel(c.M);
   a.chunk = c.chunk;
   a.rank_order = c.rank_order;
-  a.from_router = c.ru > 0 && c.early && D.shortlist != MOESPEC_STATIC && tree_router_takes(c);
+  // The router publishes the shortlist where a gate/up unit takes longer to stream than the routing needs from there to the
+  // work-unit list.  A CTA that is through with its first unit before waits for the list anyway, and streaming under the
+  // routing kernels only makes these slower; route_kernel publishes then, as for routers that do not.  us a call, published
+  // by route_kernel / by the router, by the bytes of a unit: 0.25 MB (d = 512, 64 experts, B = 32) 1 token 28.6 / 31.0, 63
+  // tokens 40.7 / 42.8; 0.5 MB (d = 1024, B = 32) 63 tokens 50.0 / 52.5, 127 tokens 54.5 / 57.2, (d = 2048, half-height units,
+  // 16 experts, B = 8) 17 tokens 35.3 / 37.0, 63 tokens 38.2 / 42.6; 0.63 MB (d = 1280, B = 32) 63 tokens 54.1 / 56.9; 0.7
+  // MB (d = 2816, half-height) 31 tokens 46.3 / 45.0, 63 tokens 48.4 / 49.2; 1 MB (d = 2048, B = 16) 63 tokens 52.2 / 51.6,
+  // (d = 4096, half-height) 58.8 / 57.8.  Up to 16 tokens nothing is gathered and the list comes sooner, so that the line
+  // lies lower: 0.25 MB (d = 1024, half-height, 128 experts) one token 30.8 / 34.0; 0.5 MB (d = 2048, half-height) one token
+  // 33.8 / 35.3 with f = 1024, but 35.8 / 33.3 with 768 and 35.1 / 33.2 (128 experts) with 512.
+  const bool short_units = (long long)c.ru * D.d <= (c.dense_all ? 96 : 160) * 1024;
+  a.from_router = c.ru > 0 && c.early && D.shortlist != MOESPEC_STATIC && tree_router_takes(c) && !short_units;
   a.dense_all = c.ru > 0 ? c.dense_all : 0;
   a.res_first = c.res_count > 0 ? c.res_first : 0;
   a.res_count = c.res_count > 0 ? c.res_count : D.n_experts;
