@@ -18,6 +18,9 @@
  *     pointers are ordinary host memory.  The library never takes ownership of a
  *     caller's buffer.  Weight, bias, hidden and out buffers are borrowed; weights
  *     and bias must stay valid and unchanged for the lifetime of the handle.
+ *     The bias is read in stream order.  The router matrix is read ahead of a
+ *     kernel in front that releases its dependents early (programmatic launch),
+ *     so such a kernel must not be the one that fills it.
  *   - verify/route calls only enqueue work on the given stream and return; they
  *     do not synchronise (the *_host variant and the get_* calls do).
  *   - One call in flight per handle: the handle owns one workspace.

@@ -209,9 +209,10 @@ __device__ __forceinline__ uint4 load_early(const void *p) {
   asm volatile("ld.global.nc.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
   return v;
 }
-__device__ __forceinline__ float load_early(const float *p) {
+// A load behind a dependency wait that stays where it is written, of data that an earlier kernel may have produced.
+__device__ __forceinline__ float load_behind(const float *p) {
   float v;
-  asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  asm volatile("ld.global.cg.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
   return v;
 }
 __device__ __forceinline__ void cluster_sync() {
@@ -1257,9 +1258,6 @@ __global__ void __maxnreg__(136) tree_router_kernel(const T *__restrict__ hidden
   // two router rows of this thread; a constant of the layer, so their start is fetched before the wait
   const T *w0 = Wr + (size_t)min(e0 + g, N - 1) * d + warp * kw + tg * 8;
   const T *w1 = Wr + (size_t)min(e0 + g + 8, N - 1) * d + warp * kw + tg * 8;
-  // the bias of the logit this thread will finish
-  const int e_bias = e0 + tid / TOK % kTreeExperts;
-  const float b0 = bias && e_bias < N ? load_early(bias + e_bias) : 0.f;
   uint4 W0[U], W1[U];
 #pragma unroll
   for (int s = 0; s < U; ++s) {
@@ -1274,6 +1272,9 @@ __global__ void __maxnreg__(136) tree_router_kernel(const T *__restrict__ hidden
   cluster_sync();        // the CTAs of the cluster have started
   pdl_wait();
   pdl_trigger();
+  // the bias of the logit this thread will finish, under the loads of the first block (before the wait: no faster)
+  const int e_bias = e0 + tid / TOK % kTreeExperts;
+  const float b0 = bias && e_bias < N ? load_behind(bias + e_bias) : 0.f;
   // a finished logit goes to the CTA of the cluster that owns its token
   auto finish_logit = [&](int tl, int e, float z) {
     if (e >= N || t0 + tl >= M) return;
