@@ -10,7 +10,8 @@
 //                        tile's last logit also runs those tokens' softmax and
 //                        top-k and adds their probabilities to the per-expert
 //                        scores (a counter, never a wait).  router_mma_kernel is
-//                        the same on the tensor cores, for larger trees.
+//                        the same on the tensor cores, for 16-bit layers of more
+//                        experts or tokens.
 //   route_kernel         eight tokens per CTA: every CTA ranks the scores itself
 //                        (shortlist; CTA 0 publishes it for the FFN kernel unless the router has),
 //                        re-routes its tokens, and the CTA that finishes last
@@ -81,7 +82,7 @@ __device__ __forceinline__ int warp_take_best(const uint32_t (&key)[W], uint32_t
 // Softmax of one token by one warp (Eq. 1, fp64); lane l owns experts l, l+32, ..., whose logits are in v (-inf beyond
 // the N-th).  The exponentials of a lane are independent chains, not branches, so that they overlap.
 template <int W>
-__device__ __forceinline__ void softmax_row(const float (&v)[W], int N, double (&p)[W]) {
+__device__ __forceinline__ void softmax_row(const float (&v)[W], double (&p)[W]) {
   float mx = -CUDART_INF_F;
 #pragma unroll
   for (int s = 0; s < W; ++s) mx = fmaxf(mx, v[s]);
@@ -95,8 +96,9 @@ __device__ __forceinline__ void softmax_row(const float (&v)[W], int N, double (
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(kFull, sum, o);
   // p / sum by one division: the quotient from the rounded reciprocal is off by an ulp at most, and the exact remainder
-  // corrects it to the rounded quotient (Markstein 1990).  A division for each p took its slow path for every p that is
-  // zero: 965 cycles for a row of 16 experts, 542 this way.
+  // corrects it to the rounded quotient (Markstein 1990).  (Where the remainder is subnormal, below p = 1e-290, a logit more
+  // than 660 under the largest, the last subnormal bit may differ.)  A division for each p took its slow path for every p
+  // that is zero: 965 cycles for a row of 16 experts, 542 this way.
   const double r = 1.0 / sum;
 #pragma unroll
   for (int s = 0; s < W; ++s) {
@@ -122,7 +124,7 @@ __device__ __forceinline__ void token_softmax(const float *zrow, int N, double *
 #pragma unroll
   for (int s = 0; s < W; ++s) v[s] = lane + 32 * s < N ? load_logit(zrow + lane + 32 * s) : -CUDART_INF_F;
   double p[W];
-  softmax_row<W>(v, N, p);
+  softmax_row<W>(v, p);
 #pragma unroll
   for (int s = 0; s < W; ++s)
     if (lane + 32 * s < N) {
@@ -524,23 +526,24 @@ cudaError_t launch_router_mma<float, 8>(const LaunchCtx &, const void *) { retur
 template <>
 cudaError_t launch_router_mma<float, 16>(const LaunchCtx &, const void *) { return cudaErrorNotSupported; }
 
-// Trees beyond 64 tokens of a 16-bit layer that tree_router_kernel does not take have their products on the tensor cores
-// all the same (d must split into eight K ranges of whole 32-element steps).
+// 16-bit layers that tree_router_kernel does not take (more than 128 experts, or 768 tokens and more) have their products on
+// the tensor cores all the same where d splits into eight K ranges of whole 32-element steps.
 static bool use_router_mma(const LaunchCtx &c) {
   static const bool off = [] { const char *v = experiment_env("MOESPEC_NO_ROUTER_MMA"); return v && v[0] == '1'; }();
-  static const int min_m = [] { const char *v = experiment_env("MOESPEC_ROUTER_MMA_MIN_M"); return v ? atoi(v) : 65; }();
-  // (also for wide routers: with N >= 128 the tensor-core kernel wins at every tree size measured)
-  return !off && is_16bit(c.desc->dtype) && (c.M >= min_m || c.desc->n_experts >= 128) && c.desc->d % 256 == 0;
+  return !off && is_16bit(c.desc->dtype) && c.desc->d % 256 == 0;
 }
 
 static cudaError_t launch_softmax_topk(const LaunchCtx &c, const float *logits, int *early_flag);
 static bool tree_router_takes(const LaunchCtx &c);
 static cudaError_t launch_router_for_tree(const LaunchCtx &c, const void *hidden);
 
-// Many tokens: logits by the 64 x 16 kernel, softmax and top-k by one warp per token.  us between events, one kernel /
-// two, 64 experts of d = 2048: 512 tokens 19.6 / 22.1 (too few CTAs), 768 23.6 / 21.6, 1024 28.8 / 21.6.  Up to 32 experts
-// the 64-expert tile is at most half full while the one kernel has few CTAs per token, so the line lies higher: d = 4096,
-// 16 experts, 768 tokens 17.7 / 21.5, 1024 19.4 / 23.5, 2048 27.6 / 25.6; 8 experts, 1024 17.4 / 19.5, 2048 23.6 / 21.5.
+// Many tokens: logits by the 64 x 16 kernel, softmax and top-k by one warp per token.  us a call, tree_router_kernel / these
+// two, d = 2048: 64 experts 300 tokens 111.1 / 114.9, 500 133.9 / 137.0, 700 166.9 / 167.5, 767 173.2 / 171.7.  With 128
+// experts the two are faster from 400 tokens on (300 143.3 / 144.1, 500 166.3 / 164.5, 767 210.2 / 202.4), but their MMAs are
+// chained on one accumulator and the logits further from 64 bits (1.7e-7 against 1.2e-7), so the line is the same there.  Up
+// to 32 experts the 64-expert tile is at most half full while router_mma_kernel has few CTAs per token, so the line lies
+// higher (us between events, router_mma_kernel / the two): d = 4096, 16 experts, 768 tokens 17.7 / 21.5, 1024 19.4 / 23.5,
+// 2048 27.6 / 25.6; 8 experts, 1024 17.4 / 19.5, 2048 23.6 / 21.5.
 static bool use_router_gemm(const LaunchCtx &c) {
   return use_router_mma(c) && c.M >= (c.desc->n_experts > 32 ? 768 : 1536) && c.desc->d % 512 == 0;
 }
@@ -561,9 +564,8 @@ cudaError_t launch_router_gemm<float>(const LaunchCtx &, const void *) { return 
 template <typename T>
 static cudaError_t launch_router_t(const LaunchCtx &c, const void *hidden) {
   if (use_router_gemm(c)) return launch_router_gemm<T>(c, hidden);
-  // sixteen warps per CTA where K splits sixteen ways into whole 32-element steps: the eight tokens of a tile
-  // then get their softmax and their top-k on separate warps (2.5 µs per layer less than eight warps at
-  // 65 to 255 tokens and for 128 experts)
+  // sixteen warps per CTA where K splits sixteen ways into whole 32-element steps: the eight tokens of a tile then get
+  // their softmax and their top-k on separate warps
   if (use_router_mma(c))
     return c.desc->d % 512 == 0 ? launch_router_mma<T, 16>(c, hidden) : launch_router_mma<T, 8>(c, hidden);
   const moespec_layer_desc &D = *c.desc;
@@ -1150,7 +1152,8 @@ __global__ void __launch_bounds__(kRouteWarps * 32) route_kernel(RouteArgs a) {
 }
 
 // Shortlist from the completed scores and union, by one CTA, for the FFN kernel's CTAs that wait for it: as
-// pick_shortlist, but nothing is kept.
+// pick_shortlist, but nothing is kept.  (Here, where the weight stream waits for the result, up to eight threads share an
+// expert: one token of 64 experts 34.4 us, 35.2 with one thread each, tree of 63 76.0 and 76.4.)
 __device__ __forceinline__ void publish_shortlist(const RouteArgs &a, unsigned long long *s_score) {
   const int tid = threadIdx.x, N = a.N;
   int gs = 0;
