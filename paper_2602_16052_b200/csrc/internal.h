@@ -68,7 +68,7 @@ struct Workspace {
   int *natcnt_acc;      // [N] number of tokens with expert i in T_k(h_t)
   int *count_acc;       // [N] number of tokens with expert i in A(t)
   unsigned *colmask;    // [N, ceil(max_M/32)] bit t of row i: expert i in A(t)
-  int *arrive;          // [max_M] arrival counters of router_topk_kernel's token tiles
+  int *arrive;          // [max_M] arrival counters of the routers' token tiles ([0]: tree_router_kernel's CTAs)
   int *arrive_route;    // [1] arrival counter of route_kernel's CTAs
   int *early_flag;      // [N] word r is 0 until the shortlist of the call is published, then (resident expert of
                         // rank r) + 1, or -1 when there are fewer (may be null)
